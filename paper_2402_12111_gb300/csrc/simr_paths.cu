@@ -9,22 +9,46 @@
 // Per path at maturity: S_T = S0 e^{x_T} (AssetPathExponential) and the payoff
 // terms of each strike.  Reduction over paths (Sec. 6): a transposed warp
 // butterfly in FP32 sums 32 paths per strike in 31 shuffle-add steps for 32
-// strikes at once, then one FP64 add per lane into per-warp shared-memory
-// accumulators; per block the warps are summed in FP64 in fixed order into a
-// partial row in global scratch, and the last block to finish (atomic ticket)
-// sums the rows in block order and normalises.  No path data touches HBM.
+// strikes at once; an item's sums go to the item's row in shared memory, the
+// block's rows are summed in FP64 in item order, and the blocks' totals on two
+// levels of atomic tickets, in block order, then normalised.  No path data
+// touches HBM.
+//
+// What bounds the kernels: the issue of their arithmetic.  A packed FMA holds both
+// FP32 pipes for two cycles and a Philox product the heavy one for four; with
+// every warp busy an SM sub-partition spends 115 cycles on 32 path-steps of
+// pricing, 88 of them on the heavy pipe.  So what counts besides the arithmetic
+// itself is that all warps stay busy to the end: with a fixed share of the paths per
+// warp the scheduler lets some warps run ahead, 4.5 of 6 warps were busy on
+// average, and one thread per sum then added 608 rows.  Items taken from a
+// counter and the two-level sums: pricing 252 steps x 2^20 paths x 32 strikes
+// 885 -> 780 us, the 5-scenario Greeks 2,510 -> 2,270 us, one strike's delta,
+// gamma and vega at 64 x 65,536 52.7 -> 43.5 us (warm calls back to back).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "simr_device.cuh"
 #include "simr_internal.h"
 #include "simr_reduce.cuh"
 
-// Tuning knobs (compile-time): resident 256-thread blocks per SM the 5-scenario
-// kernel is register-budgeted for.
-#ifndef SIMR_FD5_BLOCKS_PER_SM
-#define SIMR_FD5_BLOCKS_PER_SM 3
+// Tuning knobs (compile-time): warps per SM of the pricing and the 3- and
+// 5-scenario kernels.  Measured at 252 steps x 2^20 paths: pricing 789 / 777 /
+// 789 us at 24 / 28 / 32 warps; 5 scenarios 2,446 / 2,270 / 2,270 us at 20 / 28 / 32.
+// QE-M pricing 285 / 289 / 242 us at 24 / 28 / 32 (101 steps x 300,007 paths x 40
+// strikes: 31 batches a block).
+#ifndef SIMR_PRICE_WARPS
+#define SIMR_PRICE_WARPS 28
+#endif
+#ifndef SIMR_QEM_WARPS
+#define SIMR_QEM_WARPS 32
+#endif
+#ifndef SIMR_FD3_WARPS
+#define SIMR_FD3_WARPS 32
+#endif
+#ifndef SIMR_FD5_WARPS
+#define SIMR_FD5_WARPS 28
 #endif
 // paths per thread of the pricing (one scenario) and bump-and-revalue kernels
 #ifndef SIMR_PRICE_PPT
@@ -246,7 +270,7 @@ __device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint64_t
     for (int j = 0; j < PPT; ++j) wv[j] = w[j].z, wx[j] = w[j].w;
     step_paths<NS, NV, DYN, PPT, QEM>(L, wv, wx, v, x, c);
   }
-  if ((L.steps & 1u) && pairs >= i0) {  // odd last step (step 0 itself when steps == 1 without the split)
+  if ((L.steps & 1u) && !(NS > 1 && L.first_split && L.steps == 1)) {  // odd last step (step 0 itself when steps == 1 without the split)
     uint32_t wv[PPT], wx[PPT];
     const PhiloxCtr u = philox_ctr(pairs, L.option_index, L.rk);
 #pragma unroll
@@ -291,23 +315,30 @@ __device__ __forceinline__ void write_results(const PathLaunch& L, int k, const 
   }
 }
 
-// Fused price / Greeks kernel.  TILE = 1 (single strike) or 32 (strike tiles).
-// Dynamic shared memory: accumulators [warps][n_acc][nk_pad] (FP64), then the
-// strike constants [nk_pad] (StrikeConst), then a flag word.
-template <int NS, int NV, int TILE, bool DYN, int PPT, bool QEM>
-__global__ void __launch_bounds__(256, (NS * PPT <= 3 ? 4 : NS * PPT <= 5 ? SIMR_FD5_BLOCKS_PER_SM : 2)) heston_paths_kernel(const __grid_constant__ PathLaunch L,
-                                                           const double* __restrict__ strikes,
-                                                           PathOutputs out, double* __restrict__ partials,
-                                                           unsigned int* __restrict__ ticket) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warps = blockDim.x / kWarp;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int row = L.n_acc * L.nk_pad;
-  double* acc = reinterpret_cast<double*>(smem_raw);
-  StrikeConst* ks = reinterpret_cast<StrikeConst*>(acc + (size_t)warps * row);
-  int* s_last = reinterpret_cast<int*>(ks + L.nk_pad);
+// Warps per block, one block per SM: the register file split by what a thread of NS
+// scenarios needs.
+template <int NS, bool QEM>
+constexpr int path_warps() {
+  return NS == 1 ? (QEM ? SIMR_QEM_WARPS : SIMR_PRICE_WARPS) : NS == 3 ? SIMR_FD3_WARPS : NS == 5 ? SIMR_FD5_WARPS : 16;
+}
 
-  for (int i = threadIdx.x; i < warps * row; i += blockDim.x) acc[i] = 0.0;
+// Fused price / Greeks kernel.  TILE = 1 (single strike) or 32 (strike tiles).
+// One block per SM; its warps take the block's batches item by item (ItemPlan).
+// Dynamic shared memory: the strike constants [nk_pad] (StrikeConst), a flag word
+// and the item counter, then the items' rows of n_acc x nk_pad sums (ItemRows).
+template <int NS, int NV, int TILE, bool DYN, int PPT, bool QEM>
+__global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
+    heston_paths_kernel(const __grid_constant__ PathLaunch L, const __grid_constant__ ItemPlan I,
+                        const double* __restrict__ strikes, PathOutputs out, double* __restrict__ partials,
+                        unsigned int* __restrict__ ticket) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31;
+  StrikeConst* ks = reinterpret_cast<StrikeConst*>(smem_raw);
+  int* s_flag = reinterpret_cast<int*>(ks + L.nk_pad);
+  unsigned* s_next = reinterpret_cast<unsigned*>(s_flag + 1);
+  const ItemRows rows(s_flag + 4, I, L.n_acc * L.nk_pad);
+
+  if (threadIdx.x == 0) *s_next = 0u;
   for (int j = threadIdx.x; j < L.nk_pad; j += blockDim.x) {
     StrikeConst k{0.0f, 0.0f, 0.0f, 0.0f};
     if (j < L.n_strikes) {
@@ -321,92 +352,80 @@ __global__ void __launch_bounds__(256, (NS * PPT <= 3 ? 4 : NS * PPT <= 5 ? SIMR
   }
   __syncthreads();
 
-  double* my_acc = acc + (size_t)warp * row;
   const uint64_t per_batch = (uint64_t)kWarp * PPT;
-  const uint64_t batches = (L.path_count + per_batch - 1) / per_batch;
-  const uint64_t total_warps = (uint64_t)gridDim.x * warps;
-  for (uint64_t b = (uint64_t)blockIdx.x * warps + warp; b < batches; b += total_warps) {
-    uint64_t pth[PPT];
-    bool act[PPT];
+  const uint64_t block0 = I.batches / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, I.batches % gridDim.x);
+  const uint64_t nb = I.batches / gridDim.x + (blockIdx.x < I.batches % gridDim.x ? 1 : 0);
+  while (true) {
+    unsigned it = 0;
+    if (lane == 0) it = atomicAdd(s_next, 1u);
+    it = __shfl_sync(kFull, it, 0);
+    uint64_t b0, b1;
+    if (!item_range(I, it, nb, b0, b1)) break;
+    ItemRow my = rows.at(I, it);
+    for (uint64_t b = b0; b < b1; ++b) {
+      uint64_t pth[PPT];
+      bool act[PPT];
 #pragma unroll
-    for (int j = 0; j < PPT; ++j) {
-      const uint64_t local = b * per_batch + (uint64_t)j * kWarp + lane;
-      act[j] = local < L.path_count;
-      pth[j] = L.path_begin + local;
-    }
-    float v[PPT][NS], x[PPT][NS], c[PPT][NS];
-    simulate_ppt<NS, NV, DYN, PPT, QEM>(L, pth, v, x, c);
-    float S[PPT][NS];
-#pragma unroll
-    for (int j = 0; j < PPT; ++j)
-#pragma unroll
-      for (int s = 0; s < NS; ++s) S[j][s] = terminal_spot(L.S0, x[j][s], c[j][s]);
-
-    // accumulator list: 0 f, 1 f^2, then set Greek bits in order
-    int a = 0, r = 0;
-    for (int bit = -2; bit < kMaxGreeks; ++bit) {
-      if (bit >= 0 && !((L.greek_mask >> bit) & 1u)) continue;
-      const bool resim = bit == 2 || bit == 3 || bit >= 5;
-      const int up = resim ? L.resim_up[r] : 0, dn = resim ? L.resim_dn[r] : 0;
-      if (TILE == 1) {
-        float t = 0.0f;
-#pragma unroll
-        for (int j = 0; j < PPT; ++j) {
-          const float tj = resim ? resim_term<NS>(L, up, dn, ks[0], S[j]) : acc_term<NS>(L, bit, a, ks[0], S[j]);
-          t += act[j] ? tj : 0.0f;
-        }
-        t = warp_sum(t);
-        if (lane == 0) my_acc[a] += (double)t;
-      } else {
-        for (int t0 = 0; t0 < L.nk_pad; t0 += 32) {
-          float vals[32];
-#pragma unroll
-          for (int jj = 0; jj < 32; ++jj) {
-            const StrikeConst k = ks[t0 + jj];
-            float t = 0.0f;
-#pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-              const float tj = resim ? resim_term<NS>(L, up, dn, k, S[j]) : acc_term<NS>(L, bit, a, k, S[j]);
-              t += act[j] ? tj : 0.0f;
-            }
-            vals[jj] = t;
-          }
-          butterfly32(vals, lane);
-          my_acc[(size_t)a * L.nk_pad + t0 + lane] += (double)vals[0];
-        }
+      for (int j = 0; j < PPT; ++j) {
+        const uint64_t local = (block0 + b) * per_batch + (uint64_t)j * kWarp + lane;
+        act[j] = local < L.path_count;
+        pth[j] = L.path_begin + local;
       }
-      if (resim) ++r;
-      ++a;
+      float v[PPT][NS], x[PPT][NS], c[PPT][NS];
+      simulate_ppt<NS, NV, DYN, PPT, QEM>(L, pth, v, x, c);
+      float S[PPT][NS];
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+#pragma unroll
+        for (int s = 0; s < NS; ++s) S[j][s] = terminal_spot(L.S0, x[j][s], c[j][s]);
+
+      // accumulator list: 0 f, 1 f^2, then set Greek bits in order
+      int a = 0, r = 0;
+      for (int bit = -2; bit < kMaxGreeks; ++bit) {
+        if (bit >= 0 && !((L.greek_mask >> bit) & 1u)) continue;
+        const bool resim = bit == 2 || bit == 3 || bit >= 5;
+        const int up = resim ? L.resim_up[r] : 0, dn = resim ? L.resim_dn[r] : 0;
+        if (TILE == 1) {
+          float t = 0.0f;
+#pragma unroll
+          for (int j = 0; j < PPT; ++j) {
+            const float tj = resim ? resim_term<NS>(L, up, dn, ks[0], S[j]) : acc_term<NS>(L, bit, a, ks[0], S[j]);
+            t += act[j] ? tj : 0.0f;
+          }
+          t = warp_sum(t);
+          if (lane == 0) my.add(a, t);
+        } else {
+          for (int t0 = 0; t0 < L.nk_pad; t0 += 32) {
+            float vals[32];
+#pragma unroll
+            for (int jj = 0; jj < 32; ++jj) {
+              const StrikeConst k = ks[t0 + jj];
+              float t = 0.0f;
+#pragma unroll
+              for (int j = 0; j < PPT; ++j) {
+                const float tj = resim ? resim_term<NS>(L, up, dn, k, S[j]) : acc_term<NS>(L, bit, a, k, S[j]);
+                t += act[j] ? tj : 0.0f;
+              }
+              vals[jj] = t;
+            }
+            butterfly32(vals, lane);
+            my.add(a * L.nk_pad + t0 + lane, vals[0]);
+          }
+        }
+        if (resim) ++r;
+        ++a;
+      }
+      my.first = false;
     }
   }
   __syncthreads();
-
-  // block partial: sum the warps in order
-  double* my_row = partials + (size_t)blockIdx.x * row;
-  for (int i = threadIdx.x; i < row; i += blockDim.x) {
-    double s = 0.0;
-    for (int w = 0; w < warps; ++w) s += acc[(size_t)w * row + i];
-    my_row[i] = s;
-  }
-  __threadfence();
+  sum_item_rows(rows, I, nb);
   __syncthreads();
-  if (threadIdx.x == 0) *s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1) ? 1 : 0;
-  __syncthreads();
-  if (!*s_last) return;
-  __threadfence();
-
-  // last block: sum the partial rows in block order, then normalise per strike
-  for (int i = threadIdx.x; i < row; i += blockDim.x) {
-    double s = 0.0;
-    for (unsigned bidx = 0; bidx < gridDim.x; ++bidx) s += __ldcg(partials + (size_t)bidx * row + i);
-    acc[i] = s;
-  }
-  __syncthreads();
+  if (!sum_block_rows(rows.acc, rows.row, partials, ticket, s_flag)) return;
   for (int k = threadIdx.x; k < L.n_strikes; k += blockDim.x) {
     const double K = strikes[k];
-    write_results(L, k, acc + k, L.nk_pad, out, !(K > 0.0) || !isfinite(K));
+    write_results(L, k, rows.acc + k, L.nk_pad, out, !(K > 0.0) || !isfinite(K));
   }
-  if (threadIdx.x == 0) *ticket = 0u;
 }
 
 // Normalise sums of a sharded run: sums[k][n_acc] -> outputs.
@@ -432,32 +451,63 @@ template <int NS, int NV, int TILE, bool DYN, bool QEM = false,
           int PPT = (NS == 1 ? SIMR_PRICE_PPT : SIMR_FD_PPT)>
 cudaError_t launch_t(const PathLaunch& L, const double* strikes, const PathOutputs& out, const Scratch& s,
                      int num_sms, cudaStream_t stream, int* grid_used) {
-  const int tpb = 256, warps = tpb / kWarp;
   const size_t row = (size_t)L.n_acc * L.nk_pad;
-  const size_t smem = warps * row * sizeof(double) + L.nk_pad * sizeof(StrikeConst) + 16;
+  const size_t head = L.nk_pad * sizeof(StrikeConst) + 16;
+  const uint64_t batches = (L.path_count + (uint64_t)kWarp * PPT - 1) / ((uint64_t)kWarp * PPT);
+  const uint64_t grid = std::min<uint64_t>(num_sms, batches);  // one block per SM
+  const ItemPlan I = make_item_plan(batches, grid, path_warps<NS, QEM>(), row, kItemBytes - head);
+  const int tpb = kWarp * I.warps;
+  const size_t smem = head + item_rows_bytes(I, row);
   auto kern = heston_paths_kernel<NS, NV, TILE, DYN, PPT, QEM>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tpb, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const uint64_t batches = (L.path_count + (uint64_t)kWarp * PPT - 1) / ((uint64_t)kWarp * PPT);
-  uint64_t grid = (uint64_t)num_sms * per_sm;
-  const uint64_t need = (batches + warps - 1) / warps;
-  if (grid > need) grid = need;
-  if (grid < 1) grid = 1;
-  if ((size_t)grid * row > s.partial_doubles) return cudaErrorMemoryAllocation;
+  if ((size_t)(grid + kRowGroups) * row > s.partial_doubles) return cudaErrorMemoryAllocation;
   *grid_used = (int)grid;
-  kern<<<(unsigned)grid, tpb, smem, stream>>>(L, strikes, out, s.partials, s.ticket);
+  kern<<<(unsigned)grid, tpb, smem, stream>>>(L, I, strikes, out, s.partials, s.ticket);
   return cudaGetLastError();
 }
 
 }  // namespace
 
+ItemPlan make_item_plan(uint64_t batches, uint64_t grid, int max_warps, size_t row, size_t bytes) {
+  ItemPlan I{};
+  I.batches = batches;
+  const uint64_t q = batches / grid, most = (batches + grid - 1) / grid;  // batches of a block
+  const uint64_t fits = (bytes - row * 8) / (row * 8);                    // FP64 rows beside the totals
+  uint64_t w = std::max<uint64_t>(1, std::min<uint64_t>({(uint64_t)max_warps, fits, most}));
+  // few batches a warp: as many warps as make the rounds even (31 batches on 28
+  // warps: two rounds of 16, not 28 and 3)
+  const uint64_t rounds = (most + w - 1) / w;
+  if (rounds <= 4) w = (most + rounds - 1) / rounds;
+  I.warps = (int)w;
+  bytes -= std::max<size_t>(row, 32 * w) * 8 + 8;
+  // the fewest levels after which the rest, batch by batch in FP32 rows, fits; if
+  // none does, levels as long as the rows leave three wider FP64 items a warp
+  uint64_t rem = q;
+  while ((uint64_t)I.levels * w * row * 8 + (rem + 1) * row * 4 > bytes && I.levels < kItemLevels &&
+         rem * 3 >= 5 * w && (uint64_t)(I.levels + 4) * w * row * 8 <= bytes) {
+    const uint64_t size = rem * 3 / (5 * w);
+    I.size[I.levels] = size;
+    I.begin[I.levels] = q - rem;
+    ++I.levels;
+    rem -= size * w;
+  }
+  const uint64_t left = rem + (most - q), used = (uint64_t)I.levels * w;
+  I.tail_begin = q - rem;
+  I.tail_size = 1;
+  I.rows64 = (int32_t)used;
+  I.rows32 = (int32_t)left;
+  if ((used * 8 + left * 4) * row > bytes) {
+    const uint64_t room = bytes / (row * 8) - used;
+    I.tail_size = std::max<uint64_t>(2, (left + room - 1) / room);
+    I.rows64 = (int32_t)(used + (left + I.tail_size - 1) / I.tail_size);
+    I.rows32 = 0;
+  }
+  return I;
+}
+
 size_t paths_scratch_doubles(const PathLaunch& L, int num_sms) {
-  // at most 8 resident blocks of 256 threads per SM
-  return (size_t)num_sms * 8 * (size_t)L.n_acc * L.nk_pad;
+  return (size_t)(num_sms + kRowGroups) * (size_t)L.n_acc * L.nk_pad;
 }
 
 cudaError_t launch_paths(const PathLaunch& L, const double* strikes, const PathOutputs& out, const Scratch& s,

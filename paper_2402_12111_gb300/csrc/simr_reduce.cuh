@@ -4,6 +4,8 @@
 
 #include <cstdint>
 
+#include "simr_internal.h"
+
 namespace simr {
 namespace {
 
@@ -29,6 +31,135 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
   return v;
+}
+
+// The batches [b0, b1) of item `it` of a block that owns nb batches; false past the last.
+__device__ __forceinline__ bool item_range(const ItemPlan& I, uint32_t it, uint64_t nb, uint64_t& b0, uint64_t& b1) {
+  const uint32_t lvl = it / (uint32_t)I.warps;
+  if (lvl < (uint32_t)I.levels) {
+    b0 = I.begin[lvl] + (uint64_t)(it - lvl * I.warps) * I.size[lvl];
+    b1 = b0 + I.size[lvl];
+  } else {
+    b0 = I.tail_begin + (uint64_t)(it - (uint32_t)(I.levels * I.warps)) * I.tail_size;
+    b1 = b0 + I.tail_size;
+  }
+  if (b1 > nb) b1 = nb;
+  return b0 < nb;
+}
+
+// An item's row: the sums of its batches, added in FP64 in batch order -- or, for
+// an item of one batch, that batch's FP32 sums as they are.
+struct ItemRow {
+  double* wide;   // null for an FP32 row
+  float* narrow;
+  bool first;     // the item's first batch sets the row
+  __device__ __forceinline__ void add(int i, float t) const {
+    if (!wide)
+      narrow[i] = t;
+    else
+      wide[i] = first ? (double)t : wide[i] + (double)t;
+  }
+};
+
+// The shared memory of a block's items: FP64 rows [rows64][row], the block's
+// totals, FP32 rows [rows32][row].
+struct ItemRows {
+  double* wide;
+  double* acc;
+  float* narrow;
+  int row;
+  __device__ __forceinline__ ItemRows(void* smem, const ItemPlan& I, int row_) : row(row_) {
+    wide = reinterpret_cast<double*>(smem);
+    acc = wide + (size_t)I.rows64 * row;
+    narrow = reinterpret_cast<float*>(acc + max(row, (int)blockDim.x));
+  }
+  __device__ __forceinline__ ItemRow at(const ItemPlan& I, uint32_t it) const {
+    const uint32_t n64 = I.tail_size == 1 ? (uint32_t)(I.levels * I.warps) : 0xffffffffu;
+    return it < n64 ? ItemRow{wide + (size_t)it * row, nullptr, true}
+                    : ItemRow{nullptr, narrow + (size_t)(it - n64) * row, true};
+  }
+};
+
+// The rows of a block that owns nb batches, summed into R.acc in item order: with
+// fewer columns than threads, groups of threads sum runs of rows side by side
+// first.  All threads; rows complete on entry (after a barrier).
+__device__ __forceinline__ void sum_item_rows(const ItemRows& R, const ItemPlan& I, uint64_t nb) {
+  const int level_items = I.levels * I.warps, row = R.row;
+  const int n = level_items + (int)((nb - I.tail_begin + I.tail_size - 1) / I.tail_size);
+  const int n64 = I.tail_size == 1 ? level_items : n;
+  const int groups = max(1, min((int)blockDim.x / row, n));
+  const int per = (n + groups - 1) / groups;
+  for (int i = threadIdx.x; i < row * groups; i += blockDim.x) {
+    const int g = i / row, col = i - g * row;
+    const int r1 = min((g + 1) * per, n);
+    double s = 0.0;
+    int r = g * per;
+    for (; r < min(r1, n64); ++r) s += R.wide[(size_t)r * row + col];
+    for (; r < r1; ++r) s += (double)R.narrow[(size_t)(r - n64) * row + col];
+    R.acc[i] = s;
+  }
+  if (groups == 1) return;
+  __syncthreads();
+  for (int i = threadIdx.x; i < row; i += blockDim.x) {
+    double s = R.acc[i];
+    for (int g = 1; g < groups; ++g) s += R.acc[g * row + i];
+    R.acc[i] = s;
+  }
+}
+
+__device__ __forceinline__ double sum_rows_in_order(const double* __restrict__ p, int n, size_t row) {
+  double s = 0.0;
+  int b = 0;
+  for (; b + 8 <= n; b += 8) {  // eight loads in flight
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = __ldcg(p + (size_t)(b + k) * row);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += v[k];
+  }
+  for (; b < n; ++b) s += __ldcg(p + (size_t)b * row);
+  return s;
+}
+
+// The sum over blocks of their rows acc[0 .. row) (shared memory), in block order
+// and on two levels: the last block of a group to arrive sums the group's rows,
+// the last group's block the groups'.  True in every thread of the block that
+// ends with the totals in acc; the tickets are zero again then.  One level over
+// 608 rows took 45 us of the pricing call at 2^20 paths (one thread per column,
+// each load's latency on the path), this takes about 4.
+__device__ __forceinline__ bool sum_block_rows(double* acc, int row, double* __restrict__ partials,
+                                               unsigned int* __restrict__ ticket, int* s_flag) {
+  const int grid = gridDim.x;
+  int per = 1;
+  while (per * per < grid) ++per;
+  per = max(per, (grid + kRowGroups - 1) / kRowGroups);  // blocks per group
+  const int groups = (grid + per - 1) / per, g = blockIdx.x / per;
+  const int g0 = g * per, gn = min(per, grid - g0);
+  double* my_row = partials + (size_t)blockIdx.x * row;
+  for (int i = threadIdx.x; i < row; i += blockDim.x) my_row[i] = acc[i];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) *s_flag = atomicAdd(ticket + 1 + g, 1u) == (unsigned)gn - 1u;
+  __syncthreads();
+  if (!*s_flag) return false;
+  __threadfence();
+  double* g_row = partials + (size_t)(grid + g) * row;
+  for (int i = threadIdx.x; i < row; i += blockDim.x)
+    g_row[i] = sum_rows_in_order(partials + (size_t)g0 * row + i, gn, row);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ticket[1 + g] = 0u;
+    *s_flag = atomicAdd(ticket, 1u) == (unsigned)groups - 1u;
+  }
+  __syncthreads();
+  if (!*s_flag) return false;
+  __threadfence();
+  for (int i = threadIdx.x; i < row; i += blockDim.x)
+    acc[i] = sum_rows_in_order(partials + (size_t)grid * row + i, groups, row);
+  if (threadIdx.x == 0) *ticket = 0u;
+  __syncthreads();
+  return true;
 }
 
 struct StrikeConst {
