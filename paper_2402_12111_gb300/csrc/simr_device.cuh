@@ -228,6 +228,51 @@ __device__ __forceinline__ uint4 philox_draw(const PhiloxLane& l, const PhiloxCt
   return make_uint4(c0, c1, c2, c3);
 }
 
+// Rounds 2..9 again, for a launch whose paths all share the counter's high path
+// word phi: round 2's first product M0 (a ^ lo(M1 phi)) is then a function of the
+// step pair too, and (hi ^ rk[2][1], lo, b ^ rk[2][0], c) of every pair can be
+// formed once per block, in a shared-memory table.  15 of the 20 products and none
+// of the step pair's own are left to a path's draw (pricing 780 -> 765 us, the
+// 5-scenario Greeks 2,278 -> 2,220 us at 252 steps x 2^20 paths).
+__device__ __forceinline__ uint4 philox_pair_entry(uint32_t p, uint32_t option, uint32_t phi,
+                                                   const uint32_t (&rk)[10][2]) {
+  const PhiloxCtr u = philox_ctr(p, option, rk);
+  const uint32_t c0 = u.a ^ (kPhiloxM1 * phi);
+  return make_uint4(__umulhi(kPhiloxM0, c0) ^ rk[2][1], kPhiloxM0 * c0, u.b ^ rk[2][0], u.c);
+}
+
+__device__ __forceinline__ uint4 philox_draw_pair(const PhiloxLane& l, const uint4& e, const uint32_t (&rk)[10][2]) {
+  const uint32_t d = l.h0 ^ e.w;
+  uint32_t c0 = __umulhi(kPhiloxM1, d) ^ e.z, c1 = kPhiloxM1 * d, c2 = e.x ^ l.l0, c3 = e.y;
+#pragma unroll
+  for (int i = 3; i < 10; ++i) {
+    const uint32_t lo0 = kPhiloxM0 * c0, hi0 = __umulhi(kPhiloxM0, c0);
+    const uint32_t lo1 = kPhiloxM1 * c2, hi1 = __umulhi(kPhiloxM1, c2);
+    const uint32_t n0 = hi1 ^ c1 ^ rk[i][0];
+    const uint32_t n2 = hi0 ^ c3 ^ rk[i][1];
+    c0 = n0;
+    c1 = lo1;
+    c2 = n2;
+    c3 = lo0;
+  }
+  return make_uint4(c0, c1, c2, c3);
+}
+
+// The draws of step pair p for N paths, with the launch's table (TAB) or without.
+template <bool TAB, int N>
+__device__ __forceinline__ void philox_draws(const uint4* tab, uint32_t p, uint32_t option,
+                                             const uint32_t (&rk)[10][2], const PhiloxLane (&pl)[N], uint4 (&w)[N]) {
+  if constexpr (TAB) {
+    const uint4 e = tab[p];
+#pragma unroll
+    for (int j = 0; j < N; ++j) w[j] = philox_draw_pair(pl[j], e, rk);
+  } else {
+    const PhiloxCtr u = philox_ctr(p, option, rk);
+#pragma unroll
+    for (int j = 0; j < N; ++j) w[j] = philox_draw(pl[j], u, rk);
+  }
+}
+
 // The whole generator for one counter.
 __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                                const uint32_t (&rk)[10][2]) {
@@ -290,11 +335,12 @@ __device__ __forceinline__ float norminv_centered(float x) {
   const float p = wc < 2.5f ? norminv_central(wc) : norminv_tail(__fadd_rn(wc, 2.5f));
   return __fmul_rn(p, x);
 }
-// Two inverse normals at once (the central polynomial paired, the rare tail per lane).
-__device__ __forceinline__ float2 norminv_centered2(float2 x) {
+// Two inverse normals at once: the central polynomial paired (z valid for a lane
+// whose wc < 2.5), true when both lanes are central ...
+__device__ __forceinline__ bool norminv_try2(float2 x, float2& wc, float2& z) {
   const float2 t = p_fma(x, x, p_bc(-1.0f));
   const float2 L = make_float2(lg2_approx(fabsf(t.x)), lg2_approx(fabsf(t.y)));
-  const float2 wc = p_fma(L, p_bc(-0.69314718055994531f), p_bc(-2.5f));
+  wc = p_fma(L, p_bc(-0.69314718055994531f), p_bc(-2.5f));
   float2 p = p_bc(SIMR_S2(2.81022636e-08));
   p = p_fma(p, wc, p_bc(SIMR_S2(3.43273939e-07)));
   p = p_fma(p, wc, p_bc(SIMR_S2(-3.5233877e-06)));
@@ -304,11 +350,18 @@ __device__ __forceinline__ float2 norminv_centered2(float2 x) {
   p = p_fma(p, wc, p_bc(SIMR_S2(-0.00417768164)));
   p = p_fma(p, wc, p_bc(SIMR_S2(0.246640727)));
   p = p_fma(p, wc, p_bc(SIMR_S2(1.50140941)));
-  if (!(wc.x < 2.5f && wc.y < 2.5f)) {  // one test on the common path
-    if (!(wc.x < 2.5f)) p.x = norminv_tail(__fadd_rn(wc.x, 2.5f));
-    if (!(wc.y < 2.5f)) p.y = norminv_tail(__fadd_rn(wc.y, 2.5f));
-  }
-  return p_mul(p, x);
+  z = p_mul(p, x);
+  return wc.x < 2.5f && wc.y < 2.5f;
+}
+// ... and the rare tail lanes redone one by one.
+__device__ __forceinline__ void norminv_fix2(float2 x, float2 wc, float2& z) {
+  if (!(wc.x < 2.5f)) z.x = __fmul_rn(norminv_tail(__fadd_rn(wc.x, 2.5f)), x.x);
+  if (!(wc.y < 2.5f)) z.y = __fmul_rn(norminv_tail(__fadd_rn(wc.y, 2.5f)), x.y);
+}
+__device__ __forceinline__ float2 norminv_centered2(float2 x) {
+  float2 wc, z;
+  if (!norminv_try2(x, wc, z)) norminv_fix2(x, wc, z);  // one test on the common path
+  return z;
 }
 #undef SIMR_S2
 
@@ -381,12 +434,12 @@ __device__ __forceinline__ void qe_from_moments(float m, float s2h, float xv, fl
     qe_exp_branch(m, s2h, m2, xv, v_next, dl);
 }
 
-// Two QE variance steps: the quadratic branch paired for both lanes, then any
-// lane outside it redone by the scalar exponential branch.
-__device__ __forceinline__ void qe_from_moments2(float2 m, float2 s2h, float2 xv, float2 zv, float2& v_next,
-                                                 float2& dl) {
-  const float2 m2 = p_mul(m, m);
-  const float2 t = p_mul(m2, p_rcp(s2h));
+// Two QE variance steps: the quadratic branch paired for both lanes (true when
+// both are in it) ...
+__device__ __forceinline__ bool qe_try2(float2 m, float2 s2h, float2 zv, float2& m2, float2& t, float2& v_next,
+                                        float2& dl, float2* a_out = nullptr, float2* b2_out = nullptr) {
+  m2 = p_mul(m, m);
+  t = p_mul(m2, p_rcp(s2h));
   const float2 tm1 = p_sub(t, p_bc(1.0f));
   const float2 root = p_sqrt(p_mul(t, tm1));
   const float2 b2 = p_add(tm1, root);
@@ -395,11 +448,20 @@ __device__ __forceinline__ void qe_from_moments2(float2 m, float2 s2h, float2 xv
   const float2 bz = p_add(b, zv);
   v_next = p_mul(p_mul(a, bz), bz);
   dl = p_mul(a, p_fma(zv, p_add(bz, b), p_bc(-1.0f)));
-  const bool qx = t.x > kQuadT, qy = t.y > kQuadT;
-  if (!(qx && qy)) {  // one test on the common path
-    if (!qx) qe_exp_branch(m.x, s2h.x, m2.x, xv.x, v_next.x, dl.x);
-    if (!qy) qe_exp_branch(m.y, s2h.y, m2.y, xv.y, v_next.y, dl.y);
-  }
+  if (a_out) *a_out = a;
+  if (b2_out) *b2_out = b2;
+  return t.x > kQuadT && t.y > kQuadT;
+}
+// ... and any lane outside it redone by the scalar exponential branch.
+__device__ __forceinline__ void qe_fix2(float2 m, float2 s2h, float2 m2, float2 t, float2 xv, float2& v_next,
+                                        float2& dl) {
+  if (!(t.x > kQuadT)) qe_exp_branch(m.x, s2h.x, m2.x, xv.x, v_next.x, dl.x);
+  if (!(t.y > kQuadT)) qe_exp_branch(m.y, s2h.y, m2.y, xv.y, v_next.y, dl.y);
+}
+__device__ __forceinline__ void qe_from_moments2(float2 m, float2 s2h, float2 xv, float2 zv, float2& v_next,
+                                                 float2& dl) {
+  float2 m2, t;
+  if (!qe_try2(m, s2h, zv, m2, t, v_next, dl)) qe_fix2(m, s2h, m2, t, xv, v_next, dl);  // one test on the common path
 }
 
 // One step of the base scenario: QE variance step, then LogPricePathQE (paper
@@ -518,25 +580,25 @@ __device__ __forceinline__ bool qem_from_moments(float m, float s2h, float xv, f
   return true;  // m = 0: v' = 0, M = 1
 }
 
-// One QE-M step of the base scenario (variance step identical to step_base's);
-// where the correction does not exist the plain QE increment is taken.
+// The next variance of a QE-M path and its log-spot increment without the Z_X term
+// (variance step identical to step_base's); where the correction does not exist
+// the plain QE increment is taken.
+__device__ __forceinline__ float qem_increment(const ScenConst& c, const QemConst& q, float m, float s2h, float xv,
+                                               float zv, float v, float& vn) {
+  float dl, lam;
+  if (qem_from_moments(m, s2h, xv, zv, q.A, vn, dl, lam))
+    return __fmaf_rn(q.K2, dl, __fsub_rn(__fmaf_rn(-q.qa, __fadd_rn(v, m), q.rdt), lam));
+  float inc = __fmaf_rn(c.Cv, __fadd_rn(v, vn), c.C0);
+  inc = __fmaf_rn(-c.Cd, v, inc);
+  return __fmaf_rn(c.Cdl, dl, inc);
+}
+
+// One QE-M step of the base scenario.
 __device__ __forceinline__ void step_qem(const ScenConst& c, const QemConst& q, float xv, float zv, float zx,
                                          float& v, float& x, float& comp) {
-  float vn, dl, lam;
-  const float m = __fmaf_rn(v, c.E, c.thE);
-  const float s2h = __fmaf_rn(v, c.h1, c.h2);
-  const bool ok = qem_from_moments(m, s2h, xv, zv, q.A, vn, dl, lam);
-  const float s = __fadd_rn(v, vn);
-  float inc;
-  if (ok) {
-    inc = __fsub_rn(__fmaf_rn(-q.qa, __fadd_rn(v, m), q.rdt), lam);
-    inc = __fmaf_rn(q.K2, dl, inc);
-  } else {
-    inc = __fmaf_rn(c.Cv, s, c.C0);
-    inc = __fmaf_rn(-c.Cd, v, inc);
-    inc = __fmaf_rn(c.Cdl, dl, inc);
-  }
-  inc = __fmaf_rn(__fmul_rn(c.sK3, sqrt_approx(s)), zx, inc);
+  float vn;
+  float inc = qem_increment(c, q, __fmaf_rn(v, c.E, c.thE), __fmaf_rn(v, c.h1, c.h2), xv, zv, v, vn);
+  inc = __fmaf_rn(__fmul_rn(c.sK3, sqrt_approx(__fadd_rn(v, vn))), zx, inc);
   const float y = __fsub_rn(inc, comp);
   const float t = __fadd_rn(x, y);
   comp = __fsub_rn(__fsub_rn(t, x), y);
@@ -585,13 +647,11 @@ __device__ __forceinline__ void qem_from_moments2(float2 m, float2 s2h, float2 x
   }
 }
 
-// Two QE-M steps (two paths on the same constants) in packed FP32, lane for
-// lane step_qem.
-__device__ __forceinline__ void step_qem2(const ScenConst& c, const QemConst& q, float2 xv, float2 zv, float2 zx,
-                                          float2& v, float2& x, float2& comp) {
-  const float2 m = p_fma(v, p_bc(c.E), p_bc(c.thE));
-  const float2 s2h = p_fma(v, p_bc(c.h1), p_bc(c.h2));
-  float2 vn, dl, lam;
+// The next variance of two QE-M paths (on the same constants) and their log-spot
+// increments without the Z_X term, lane for lane step_qem's.
+__device__ __forceinline__ float2 qem_increment2(const ScenConst& c, const QemConst& q, float2 m, float2 s2h,
+                                                 float2 xv, float2 zv, float2 v, float2& vn) {
+  float2 dl, lam;
   bool okx, oky;
   qem_from_moments2(m, s2h, xv, zv, p_bc(q.A), vn, dl, lam, okx, oky);
   const float2 s = p_add(v, vn);
@@ -616,12 +676,29 @@ __device__ __forceinline__ void step_qem2(const ScenConst& c, const QemConst& q,
     }
     inc = make_float2(r[0], r[1]);
   }
-  inc = p_fma(p_mul(p_bc(c.sK3), p_sqrt(s)), zx, inc);
+  return inc;
+}
+
+// The end of a step of two paths: the Z_X term, x (Kahan-compensated), v.
+__device__ __forceinline__ void advance2(const ScenConst& c, float2 inc, float2 zx, float2 vn, float2& v, float2& x,
+                                         float2& comp) {
+  inc = p_fma(p_mul(p_bc(c.sK3), p_sqrt(p_add(v, vn))), zx, inc);
   const float2 y = p_sub(inc, comp);
-  const float2 t2 = p_add(x, y);
-  comp = p_sub(p_sub(t2, x), y);
-  x = t2;
+  const float2 t = p_add(x, y);
+  comp = p_sub(p_sub(t, x), y);
+  x = t;
   v = vn;
+}
+
+// Two QE-M steps (two paths on the same constants) in packed FP32, lane for
+// lane step_qem.
+__device__ __forceinline__ void step_qem2(const ScenConst& c, const QemConst& q, float2 xv, float2 zv, float2 zx,
+                                          float2& v, float2& x, float2& comp) {
+  const float2 m = p_fma(v, p_bc(c.E), p_bc(c.thE));
+  const float2 s2h = p_fma(v, p_bc(c.h1), p_bc(c.h2));
+  float2 vn;
+  const float2 inc = qem_increment2(c, q, m, s2h, xv, zv, v, vn);
+  advance2(c, inc, zx, vn, v, x, comp);
 }
 
 // One step of the base scenario under scheme QEM (false: QE) with the CRN
@@ -920,6 +997,117 @@ __device__ __forceinline__ void simulate_two(const ScenConst& c, uint32_t steps,
       else
         step_base2<false>(c, xv, zv, zx, v, x, comp);
     }
+  }
+}
+
+// The draws of one time step of two paths: 2 U_V - 1, Z_V, Z_X.
+struct Draw2 {
+  float2 xv, zv, zx;
+};
+struct DrawFix2 {  // what a tail normal is redone from
+  float2 xx, wcv, wcx;
+};
+
+__device__ __forceinline__ bool draw_try2(uint32_t wv0, uint32_t wv1, uint32_t wx0, uint32_t wx1, Draw2& d,
+                                          DrawFix2& f) {
+  d.xv = centered_uniform2(wv0, wv1);
+  f.xx = centered_uniform2(wx0, wx1);
+  const bool a = norminv_try2(d.xv, f.wcv, d.zv);
+  return norminv_try2(f.xx, f.wcx, d.zx) && a;
+}
+__device__ __forceinline__ void draw_fix2(Draw2& d, const DrawFix2& f) {
+  norminv_fix2(d.xv, f.wcv, d.zv);
+  norminv_fix2(f.xx, f.wcx, d.zx);
+}
+
+// One time step of two paths from its draws `d`, and the draws `dn` of the step
+// after it, from that step's words.  The two are independent, and everything off
+// the common path -- a tail among the next normals, a lane outside the quadratic
+// branch (QE-M: or with |u| >= 1/8) -- is redone behind one test, so the scheduler
+// sees the variance step's chain, the next normals and the generator's rounds
+// around them as one block.
+template <bool QEM>
+__device__ __forceinline__ void pipe_step2(const ScenConst& c, const QemConst& q, const Draw2& d, uint32_t wv0,
+                                           uint32_t wv1, uint32_t wx0, uint32_t wx1, Draw2& dn, float2& v, float2& x,
+                                           float2& comp) {
+  const float2 m = p_fma(v, p_bc(c.E), p_bc(c.thE));
+  const float2 s2h = p_fma(v, p_bc(c.h1), p_bc(c.h2));
+  float2 vn, dl, m2, t, a, b2, inc;
+  DrawFix2 f;
+  bool fx = true, fy = true;  // QE-M: the lane's fast values hold
+  bool common = qe_try2(m, s2h, d.zv, m2, t, vn, dl, &a, &b2);
+  if constexpr (QEM) {  // qem_from_moments2's quadratic branch, g by its series
+    const float2 Aa = p_mul(p_bc(q.A), a);
+    const float2 u = p_mul(p_bc(2.0f), Aa);
+    float2 g = p_fma(u, p_bc(0.125f), p_bc(0.14285714285714285f));
+    g = p_fma(u, g, p_bc(0.16666666666666666f));
+    g = p_fma(u, g, p_bc(0.2f));
+    g = p_fma(u, g, p_bc(0.25f));
+    g = p_fma(u, g, p_bc(0.33333333333333333f));
+    g = p_fma(u, g, p_bc(0.5f));
+    g = p_mul(p_mul(u, u), g);
+    const float2 lam = p_fma(p_bc(0.5f), g, p_mul(p_mul(p_mul(p_mul(p_bc(2.0f), Aa), Aa), b2), p_rcp(p_sub(p_bc(1.0f), u))));
+    inc = p_sub(p_fma(p_bc(-q.qa), p_add(v, m), p_bc(q.rdt)), lam);
+    inc = p_fma(p_bc(q.K2), dl, inc);
+    fx = t.x > kQuadT && fabsf(u.x) < 0.125f;
+    fy = t.y > kQuadT && fabsf(u.y) < 0.125f;
+    common = fx && fy;
+  }
+  const bool central = draw_try2(wv0, wv1, wx0, wx1, dn, f);
+  if (!(common && central)) {
+    draw_fix2(dn, f);
+    if constexpr (QEM) {
+      if (!fx) inc.x = qem_increment(c, q, m.x, s2h.x, d.xv.x, d.zv.x, v.x, vn.x);
+      if (!fy) inc.y = qem_increment(c, q, m.y, s2h.y, d.xv.y, d.zv.y, v.y, vn.y);
+    } else {
+      qe_fix2(m, s2h, m2, t, d.xv, vn, dl);
+    }
+  }
+  if constexpr (!QEM) {
+    inc = p_fma(p_bc(c.Cv), p_add(v, vn), p_bc(c.C0));
+    inc = p_fma(p_bc(-c.Cd), v, inc);
+    inc = p_fma(p_bc(c.Cdl), dl, inc);
+  }
+  advance2(c, inc, d.zx, vn, v, x, comp);
+}
+
+// Two paths of one scenario in lockstep, simulate_two's values: the arithmetic of
+// simulate_one paired lane for lane, software-pipelined -- while a step's variance
+// chain runs, the next step's normals and the next pair's Philox rounds are
+// computed.  after(n) runs after step n.  A step of one warp alone takes 470 cycles
+// instead of 710; with every sub-partition full the rate is the issue's either way.
+template <bool QEM, bool TAB, class After>
+__device__ __forceinline__ void simulate_two_pipe(const ScenConst& c, uint32_t steps, uint32_t option,
+                                                  const uint32_t (&rk)[10][2], const uint4* tab, uint64_t path0,
+                                                  uint64_t path1, float2& v, float2& x, float2& comp,
+                                                  const QemConst& q, After&& after) {
+  const PhiloxLane pl[2] = {philox_lane(path0, rk), philox_lane(path1, rk)};
+  v = make_float2(c.v0, c.v0);
+  x = make_float2(0.0f, 0.0f);
+  comp = make_float2(0.0f, 0.0f);
+  uint4 w[2];
+  philox_draws<TAB, 2>(tab, 0u, option, rk, pl, w);
+  Draw2 da, db;
+  DrawFix2 f;
+  if (!draw_try2(w[0].x, w[1].x, w[0].y, w[1].y, da, f)) draw_fix2(da, f);
+  const uint32_t pairs = steps >> 1;
+#pragma unroll 1
+  for (uint32_t i = 0; i < pairs; ++i) {
+    uint4 n[2];
+    philox_draws<TAB, 2>(tab, i + 1, option, rk, pl, n);  // (one pair past the last step is drawn and not used)
+    pipe_step2<QEM>(c, q, da, w[0].z, w[1].z, w[0].w, w[1].w, db, v, x, comp);
+    after(2 * i);
+    pipe_step2<QEM>(c, q, db, n[0].x, n[1].x, n[0].y, n[1].y, da, v, x, comp);
+    after(2 * i + 1);
+    w[0] = n[0];
+    w[1] = n[1];
+  }
+  if (steps & 1u) {
+    if constexpr (QEM)
+      step_qem2(c, q, da.xv, da.zv, da.zx, v, x, comp);
+    else
+      step_base2<false>(c, da.xv, da.zv, da.zx, v, x, comp);
+    after(steps - 1);
   }
 }
 

@@ -42,6 +42,7 @@ struct PathLaunch {
   double disc;            // e^{-rT}
   double paths_total;     // denominator of the mean
   double denom[kMaxGreeks];  // per Greek: bump denominator (sign folded in)
+  int32_t pair_table;     // entries of the step pairs' counter table in shared memory, 0: none
   int32_t raw_sums;       // 1: write raw sums instead of normalised results
   int32_t scheme;         // 0: QE; 1: QE-M
   QemConst qm;            // QE-M constants of the base scenario

@@ -39,7 +39,7 @@
 // QE-M pricing 285 / 289 / 242 us at 24 / 28 / 32 (101 steps x 300,007 paths x 40
 // strikes: 31 batches a block).
 #ifndef SIMR_PRICE_WARPS
-#define SIMR_PRICE_WARPS 28
+#define SIMR_PRICE_WARPS 24
 #endif
 #ifndef SIMR_QEM_WARPS
 #define SIMR_QEM_WARPS 32
@@ -225,9 +225,9 @@ __device__ __forceinline__ void step0_all(const PathLaunch& L, uint32_t w_v, uin
 // PPT paths per thread, simulated step by step in lockstep: independent
 // dependency chains the scheduler can interleave (instruction-level
 // parallelism at the same occupancy).
-template <int NS, int NV, bool DYN, int PPT, bool QEM = false>
-__device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint64_t (&path)[PPT], float (&v)[PPT][NS],
-                                             float (&x)[PPT][NS], float (&c)[PPT][NS]) {
+template <bool TAB, int NS, int NV, bool DYN, int PPT, bool QEM = false>
+__device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint4* tab, const uint64_t (&path)[PPT],
+                                             float (&v)[PPT][NS], float (&x)[PPT][NS], float (&c)[PPT][NS]) {
 #pragma unroll
   for (int j = 0; j < PPT; ++j) {
 #pragma unroll
@@ -244,9 +244,7 @@ __device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint64_t
   uint32_t i0 = 0;
   if (NS > 1 && L.first_split) {
     uint4 w[PPT];
-    const PhiloxCtr u = philox_ctr(0u, L.option_index, L.rk);
-#pragma unroll
-    for (int j = 0; j < PPT; ++j) w[j] = philox_draw(pl[j], u, L.rk);
+    philox_draws<TAB, PPT>(tab, 0u, L.option_index, L.rk, pl, w);
 #pragma unroll
     for (int j = 0; j < PPT; ++j) step0_all<NS, DYN, QEM>(L, w[j].x, w[j].y, v[j], x[j], c[j]);
     if (L.steps > 1) {
@@ -260,9 +258,7 @@ __device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint64_t
   for (uint32_t i = i0; i < pairs; ++i) {
     uint4 w[PPT];
     uint32_t wv[PPT], wx[PPT];
-    const PhiloxCtr u = philox_ctr(i, L.option_index, L.rk);
-#pragma unroll
-    for (int j = 0; j < PPT; ++j) w[j] = philox_draw(pl[j], u, L.rk);
+    philox_draws<TAB, PPT>(tab, i, L.option_index, L.rk, pl, w);
 #pragma unroll
     for (int j = 0; j < PPT; ++j) wv[j] = w[j].x, wx[j] = w[j].y;
     step_paths<NS, NV, DYN, PPT, QEM>(L, wv, wx, v, x, c);
@@ -271,14 +267,11 @@ __device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint64_t
     step_paths<NS, NV, DYN, PPT, QEM>(L, wv, wx, v, x, c);
   }
   if ((L.steps & 1u) && !(NS > 1 && L.first_split && L.steps == 1)) {  // odd last step (step 0 itself when steps == 1 without the split)
+    uint4 w[PPT];
     uint32_t wv[PPT], wx[PPT];
-    const PhiloxCtr u = philox_ctr(pairs, L.option_index, L.rk);
+    philox_draws<TAB, PPT>(tab, pairs, L.option_index, L.rk, pl, w);
 #pragma unroll
-    for (int j = 0; j < PPT; ++j) {
-      const uint4 w = philox_draw(pl[j], u, L.rk);
-      wv[j] = w.x;
-      wx[j] = w.y;
-    }
+    for (int j = 0; j < PPT; ++j) wv[j] = w[j].x, wx[j] = w[j].y;
     step_paths<NS, NV, DYN, PPT, QEM>(L, wv, wx, v, x, c);
   }
 }
@@ -322,10 +315,17 @@ constexpr int path_warps() {
   return NS == 1 ? (QEM ? SIMR_QEM_WARPS : SIMR_PRICE_WARPS) : NS == 3 ? SIMR_FD3_WARPS : NS == 5 ? SIMR_FD5_WARPS : 16;
 }
 
+// Whether the kernel of NS scenarios has a loop for the step pairs' counter table:
+// not with 11 and more, nor the QE-M bumps, whose arithmetic hides what it saves.
+template <int NS, bool QEM>
+constexpr bool path_table() {
+  return NS == 1 || (NS <= 5 && !QEM);
+}
+
 // Fused price / Greeks kernel.  TILE = 1 (single strike) or 32 (strike tiles).
 // One block per SM; its warps take the block's batches item by item (ItemPlan).
 // Dynamic shared memory: the strike constants [nk_pad] (StrikeConst), a flag word
-// and the item counter, then the items' rows of n_acc x nk_pad sums (ItemRows).
+// and the item counter, the step pairs' counter table, then the items' rows of n_acc x nk_pad sums (ItemRows).
 template <int NS, int NV, int TILE, bool DYN, int PPT, bool QEM>
 __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
     heston_paths_kernel(const __grid_constant__ PathLaunch L, const __grid_constant__ ItemPlan I,
@@ -336,9 +336,12 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
   StrikeConst* ks = reinterpret_cast<StrikeConst*>(smem_raw);
   int* s_flag = reinterpret_cast<int*>(ks + L.nk_pad);
   unsigned* s_next = reinterpret_cast<unsigned*>(s_flag + 1);
-  const ItemRows rows(s_flag + 4, I, L.n_acc * L.nk_pad);
+  uint4* tab = L.pair_table ? reinterpret_cast<uint4*>(s_flag + 4) : nullptr;
+  const ItemRows rows(s_flag + 4 + 4 * L.pair_table, I, L.n_acc * L.nk_pad);
 
   if (threadIdx.x == 0) *s_next = 0u;
+  for (int p = threadIdx.x; p < L.pair_table; p += blockDim.x)
+    tab[p] = philox_pair_entry(p, L.option_index, (uint32_t)(L.path_begin >> 32), L.rk);
   for (int j = threadIdx.x; j < L.nk_pad; j += blockDim.x) {
     StrikeConst k{0.0f, 0.0f, 0.0f, 0.0f};
     if (j < L.n_strikes) {
@@ -352,6 +355,7 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
   }
   __syncthreads();
 
+  constexpr bool USE_TAB = path_table<NS, QEM>();
   const uint64_t per_batch = (uint64_t)kWarp * PPT;
   const uint64_t block0 = I.batches / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, I.batches % gridDim.x);
   const uint64_t nb = I.batches / gridDim.x + (blockIdx.x < I.batches % gridDim.x ? 1 : 0);
@@ -372,7 +376,23 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
         pth[j] = L.path_begin + local;
       }
       float v[PPT][NS], x[PPT][NS], c[PPT][NS];
-      simulate_ppt<NS, NV, DYN, PPT, QEM>(L, pth, v, x, c);
+      if constexpr (NS == 1 && PPT == 2) {
+        float2 v2, x2, c2;
+        if (tab)
+          simulate_two_pipe<QEM, true>(L.sc[0], L.steps, L.option_index, L.rk, tab, pth[0], pth[1], v2, x2, c2, L.qm,
+                                       [](uint32_t) {});
+        else
+          simulate_two_pipe<QEM, false>(L.sc[0], L.steps, L.option_index, L.rk, tab, pth[0], pth[1], v2, x2, c2, L.qm,
+                                        [](uint32_t) {});
+        x[0][0] = x2.x;
+        x[1][0] = x2.y;
+        c[0][0] = c2.x;
+        c[1][0] = c2.y;
+      } else if (USE_TAB && tab) {
+        simulate_ppt<USE_TAB, NS, NV, DYN, PPT, QEM>(L, tab, pth, v, x, c);
+      } else {
+        simulate_ppt<false, NS, NV, DYN, PPT, QEM>(L, nullptr, pth, v, x, c);
+      }
       float S[PPT][NS];
 #pragma unroll
       for (int j = 0; j < PPT; ++j)
@@ -442,17 +462,29 @@ __global__ void __launch_bounds__(256) heston_terminal_kernel(const __grid_const
   if (i >= L.path_count) return;
   float v[1][1], x[1][1], c[1][1];
   const uint64_t pth[1] = {L.path_begin + i};
-  simulate_ppt<1, 0, false, 1, QEM>(L, pth, v, x, c);
+  simulate_ppt<false, 1, 0, false, 1, QEM>(L, nullptr, pth, v, x, c);
   x_T[i] = x[0][0] - c[0][0];
   if (v_T) v_T[i] = v[0][0];
 }
 
+// Entries of the shared-memory table of step-pair counters: one per pair and one
+// past the last, which a pipelined loop reads; none where the paths cross a
+// multiple of 2^32 (their high words differ), or past 32 KB (4,092 steps), which
+// the items' rows need more.
+int pair_table_entries(const PathLaunch& L) {
+  const uint64_t n = (uint64_t)L.steps / 2 + 2;
+  const bool one_high_word = (L.path_begin >> 32) == ((L.path_begin + L.path_count - 1) >> 32);
+  return one_high_word && n <= 2048 ? (int)n : 0;
+}
+
 template <int NS, int NV, int TILE, bool DYN, bool QEM = false,
           int PPT = (NS == 1 ? SIMR_PRICE_PPT : SIMR_FD_PPT)>
-cudaError_t launch_t(const PathLaunch& L, const double* strikes, const PathOutputs& out, const Scratch& s,
+cudaError_t launch_t(const PathLaunch& L0, const double* strikes, const PathOutputs& out, const Scratch& s,
                      int num_sms, cudaStream_t stream, int* grid_used) {
+  PathLaunch L = L0;
+  L.pair_table = path_table<NS, QEM>() ? pair_table_entries(L0) : 0;
   const size_t row = (size_t)L.n_acc * L.nk_pad;
-  const size_t head = L.nk_pad * sizeof(StrikeConst) + 16;
+  const size_t head = L.nk_pad * sizeof(StrikeConst) + 16 + L.pair_table * sizeof(uint4);
   const uint64_t batches = (L.path_count + (uint64_t)kWarp * PPT - 1) / ((uint64_t)kWarp * PPT);
   const uint64_t grid = std::min<uint64_t>(num_sms, batches);  // one block per SM
   const ItemPlan I = make_item_plan(batches, grid, path_warps<NS, QEM>(), row, kItemBytes - head);
