@@ -24,6 +24,7 @@
 // in the pricing kernel.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "simr_device.cuh"
@@ -57,8 +58,7 @@ inline size_t adjoint_smem_bytes_t(const PathLaunch& L, const AdjConst& A, int t
 // strike's payoff f, f^2, and the in-the-money weight w (S_T for a call above
 // its strike, -S_T for a put below) alone and times each derivative; FP32 over
 // the warp's paths.  out[0..8]: f, f^2, w, w dx/dv0 .. w dx/drho, the signed
-// in-the-money indicator (the S0 column is w / S0, scaled when added to the FP64
-// sums; the r column e^{-rT} T K times the indicator's mean, see adj_term).
+// in-the-money indicator (the S0 column is w / S0, scaled with the totals; the r column e^{-rT} T K times the indicator's mean, see adj_term).
 template <int PPT>
 __device__ __forceinline__ void strike_tile_terms(bool put, float K, const float (&S)[PPT], const bool (&act)[PPT],
                                                   const float (&g)[PPT][5], float (&out)[kAdjAcc]) {
@@ -87,30 +87,51 @@ __device__ __forceinline__ void strike_tile_terms(bool put, float K, const float
   }
 }
 
-// Minimum resident blocks per SM asked of the register allocator: 5 for global
-// segments (one segment of the whole path: 4-5% faster than its own choice, 7%
-// faster than 4), 4 for shared-memory segments (which hold a block's segment
-// buffers, 12 k bytes per thread, so that longer segments leave room for 4
-// blocks at most: 11% faster at k = 32 and 1% at k = 16 than with 5).
-#ifndef SIMR_ADJ_MINB_GSEG
-#define SIMR_ADJ_MINB_GSEG 5
-#endif
+// Price, standard error and the seven derivatives per strike from the totals
+// acc[9][nk_pad] (shared memory; s0_scale: what the S0 column's sums still lack).
+__device__ __forceinline__ void write_adjoint(const PathLaunch& L, const AdjConst& A,
+                                              const double* __restrict__ strikes, const double* acc, double s0_scale,
+                                              const AdjOutputs& out) {
+  const double inv_n = 1.0 / L.paths_total;
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
+  for (int kk = threadIdx.x; kk < L.n_strikes; kk += blockDim.x) {
+    const double K = strikes[kk];
+    const bool bad = !(K > 0.0) || !isfinite(K);
+    const double mean = acc[kk] * inv_n;
+    const double price = L.disc * mean;
+    out.price[kk] = bad ? nan : price;
+    if (out.stderr_) {
+      const double n = L.paths_total;
+      const double var = n > 1.0 ? (acc[L.nk_pad + kk] * inv_n - mean * mean) / (n - 1.0) : 0.0;
+      out.stderr_[kk] = bad ? nan : L.disc * sqrt(var > 0.0 ? var : 0.0);
+    }
+    for (int c7 = 0; c7 < 7; ++c7) {
+      double gsum = L.disc * acc[(size_t)(2 + c7) * L.nk_pad + kk] * inv_n;
+      if (c7 == 0) gsum *= s0_scale;
+      // e^{-rT} T K E[indicator] with the FP32 T and K the paths use (as the book does)
+      if (c7 == 6) gsum *= (double)A.T * (double)(float)K;
+      out.grad[(size_t)kk * 7 + c7] = bad ? nan : gsum;
+    }
+  }
+}
+
+// Minimum resident blocks per SM asked of the register allocator: 4, which is what
+// the segment buffers (12 k bytes per thread) leave room for from k = 16 on (11%
+// faster at k = 32 and 1% at k = 16 than with 5).
 #ifndef SIMR_ADJ_MINB_SMEM
 #define SIMR_ADJ_MINB_SMEM 4
 #endif
 
-// GSEG: the segment buffers in global memory, [3 k][grid threads] (for a
-// segment too long for shared memory, in particular one segment of the whole
-// path: no forward pass).
+// Segments in shared memory (an explicit checkpoint interval).
 // QEM: the QE-M log-spot step (the launch's scheme 1), differentiated one step
 // at a time.
-template <int TILE, int PPT, bool RACC, bool GSEG, bool QEM>
-__global__ void __launch_bounds__(128, GSEG ? SIMR_ADJ_MINB_GSEG : SIMR_ADJ_MINB_SMEM) heston_adjoint_kernel(const __grid_constant__ PathLaunch L,
+template <int TILE, int PPT, bool RACC, bool QEM>
+__global__ void __launch_bounds__(128, SIMR_ADJ_MINB_SMEM) heston_adjoint_kernel(const __grid_constant__ PathLaunch L,
                                                              const __grid_constant__ AdjConst A,
                                                              const double* __restrict__ strikes, AdjOutputs out,
                                                              double* __restrict__ partials,
                                                              unsigned int* __restrict__ ticket,
-                                                             float* __restrict__ gckpt, float* __restrict__ gseg) {
+                                                             float* __restrict__ gckpt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warps = blockDim.x / kWarp;
   const int bd = blockDim.x;
@@ -157,13 +178,8 @@ __global__ void __launch_bounds__(128, GSEG ? SIMR_ADJ_MINB_GSEG : SIMR_ADJ_MINB
       pth[j] = L.path_begin + local;
     }
     float x[PPT], comp[PPT], g[PPT][5], S[PPT];
-    if constexpr (GSEG)
-      path_adjoint_ppt<PPT, SegGlobal, true, QEM>(
-          L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
-          SegGlobal{gseg, (long long)blockIdx.x * bd + tid, A.ckpt_every, (long long)ck_stride}, x, comp, g, L.qm);
-    else
-      path_adjoint_ppt<PPT, SegShared, true, QEM>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
-                                                  SegShared{sbuf, A.ckpt_every}, x, comp, g, L.qm);
+    path_adjoint_ppt<PPT, SegShared, true, QEM>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
+                                                SegShared{sbuf, A.ckpt_every}, x, comp, g, L.qm);
 #pragma unroll
     for (int j = 0; j < PPT; ++j) S[j] = terminal_spot(L.S0, x[j], comp[j]);
 
@@ -186,64 +202,119 @@ __global__ void __launch_bounds__(128, GSEG ? SIMR_ADJ_MINB_GSEG : SIMR_ADJ_MINB
         float t[kAdjAcc];
         strike_tile_terms<PPT>(put, ks[t0 + lane].K, S, act, g, t);
         double* row = my_acc + t0 + lane;
-        row[0] += (double)t[0];
-        row[(size_t)L.nk_pad] += (double)t[1];
-        row[(size_t)2 * L.nk_pad] += (double)t[2] * (double)A.invS0;
 #pragma unroll
-        for (int a = 3; a < kAdjAcc; ++a) row[(size_t)a * L.nk_pad] += (double)t[a];
+        for (int a = 0; a < kAdjAcc; ++a) row[(size_t)a * L.nk_pad] += (double)t[a];
       }
     }
   }
   __syncthreads();
   if (RACC) {  // the segment buffers are free now: spill the lanes' sums into the rows
-    // racc[2] holds the weights w: the S0 column is w / S0
-    my_acc[lane] = racc[0];
-    my_acc[(size_t)L.nk_pad + lane] = racc[1];
-    my_acc[(size_t)2 * L.nk_pad + lane] = racc[2] * (double)A.invS0;
 #pragma unroll
-    for (int a = 3; a < kAdjAcc; ++a) my_acc[(size_t)a * L.nk_pad + lane] = racc[a];
+    for (int a = 0; a < kAdjAcc; ++a) my_acc[(size_t)a * L.nk_pad + lane] = racc[a];
     __syncthreads();
   }
 
-  double* my_row = partials + (size_t)blockIdx.x * row;
   for (int i = threadIdx.x; i < row; i += blockDim.x) {
-    double s = 0.0;
-    for (int w = 0; w < warps; ++w) s += acc[(size_t)w * row + i];
-    my_row[i] = s;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) *s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1) ? 1 : 0;
-  __syncthreads();
-  if (!*s_last) return;
-  __threadfence();
-  for (int i = threadIdx.x; i < row; i += blockDim.x) {
-    double s = 0.0;
-    for (unsigned b = 0; b < gridDim.x; ++b) s += __ldcg(partials + (size_t)b * row + i);
+    double s = acc[i];
+    for (int w = 1; w < warps; ++w) s += acc[(size_t)w * row + i];
     acc[i] = s;
   }
   __syncthreads();
-  const double inv_n = 1.0 / L.paths_total;
-  const double nan = __longlong_as_double(0x7ff8000000000000ll);
-  for (int kk = threadIdx.x; kk < L.n_strikes; kk += blockDim.x) {
-    const double K = strikes[kk];
-    const bool bad = !(K > 0.0) || !isfinite(K);
-    const double mean = acc[kk] * inv_n;
-    const double price = L.disc * mean;
-    out.price[kk] = bad ? nan : price;
-    if (out.stderr_) {
-      const double n = L.paths_total;
-      const double var = n > 1.0 ? (acc[L.nk_pad + kk] * inv_n - mean * mean) / (n - 1.0) : 0.0;
-      out.stderr_[kk] = bad ? nan : L.disc * sqrt(var > 0.0 ? var : 0.0);
+  if (!sum_block_rows(acc, row, partials, ticket, s_last)) return;
+  write_adjoint(L, A, strikes, acc, TILE == 1 ? 1.0 : (double)A.invS0, out);  // (as below)
+}
+
+// Warps per SM of the kernel below (QE-M: its reverse step needs fewer registers).
+#ifndef SIMR_ADJ_WARPS
+#define SIMR_ADJ_WARPS 24
+#endif
+#ifndef SIMR_ADJ_QEM_WARPS
+#define SIMR_ADJ_QEM_WARPS 28
+#endif
+
+// Segments in global memory, [3 k][grid threads] (a segment too long for shared
+// memory, in particular one segment of the whole path: no forward pass).  One block
+// per SM, its warps taking 32-path batches item by item (ItemPlan), each item's nine
+// sums per strike in the item's own row.  Issue-bound (187 warp instructions per
+// path-step, 33 of them packed).  252 steps x 2^20 paths x 32 strikes: 2,072 us with
+// five blocks of 128 that strode over the batches (and one thread per sum over 760
+// block rows at the end), 1,740 with items at 20 warps, 1,598 at 24 (80 registers;
+// 28 and 32 warps spill: 2,040 and 2,080); QE-M 948 -> 680 us at 2^18 paths.
+template <int TILE, bool QEM>
+__global__ void __launch_bounds__(kWarp * (QEM ? SIMR_ADJ_QEM_WARPS : SIMR_ADJ_WARPS), 1)
+    heston_adjoint_seg_kernel(const __grid_constant__ PathLaunch L, const __grid_constant__ AdjConst A,
+                              const __grid_constant__ ItemPlan I, const double* __restrict__ strikes, AdjOutputs out,
+                              double* __restrict__ partials, unsigned int* __restrict__ ticket,
+                              float* __restrict__ gckpt, float* __restrict__ gseg) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int bd = blockDim.x, lane = threadIdx.x & 31, tid = threadIdx.x;
+  StrikeConst* ks = reinterpret_cast<StrikeConst*>(smem_raw);
+  int* s_flag = reinterpret_cast<int*>(ks + L.nk_pad);
+  unsigned* s_next = reinterpret_cast<unsigned*>(s_flag + 1);
+  uint4* tab = L.pair_table ? reinterpret_cast<uint4*>(s_flag + 4) : nullptr;
+  const ItemRows rows(s_flag + 4 + 4 * L.pair_table, I, kAdjAcc * L.nk_pad);
+  // checkpoints: this thread's column of a [slot][grid threads] global array
+  float* ck = gckpt + (int)blockIdx.x * bd + tid;
+  const int ck_stride = (int)(gridDim.x * blockDim.x);
+  if (tid == 0) *s_next = 0u;
+  for (int p = tid; p < L.pair_table; p += bd)
+    tab[p] = philox_pair_entry(p, L.option_index, (uint32_t)(L.path_begin >> 32), L.rk);
+  for (int j = tid; j < L.nk_pad; j += bd) {
+    StrikeConst k{0.0f, 0.0f, 0.0f, 0.0f};
+    if (j < L.n_strikes) {
+      const double K = strikes[j];
+      if (!(K > 0.0) || !isfinite(K)) atomicOr(out.status, 1);
+      k.K = (float)K;
     }
-    for (int c7 = 0; c7 < 7; ++c7) {
-      double gsum = L.disc * acc[(size_t)(2 + c7) * L.nk_pad + kk] * inv_n;
-      // e^{-rT} T K E[indicator] with the FP32 T and K the paths use (as the book does)
-      if (c7 == 6) gsum *= (double)A.T * (double)(float)K;
-      out.grad[(size_t)kk * 7 + c7] = bad ? nan : gsum;
+    ks[j] = k;
+  }
+  __syncthreads();
+
+  const bool put = L.is_put != 0;
+  const uint64_t block0 = I.batches / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, I.batches % gridDim.x);
+  const uint64_t nb = I.batches / gridDim.x + (blockIdx.x < I.batches % gridDim.x ? 1 : 0);
+  while (true) {
+    unsigned it = 0;
+    if (lane == 0) it = atomicAdd(s_next, 1u);
+    it = __shfl_sync(kFull, it, 0);
+    uint64_t b0, b1;
+    if (!item_range(I, it, nb, b0, b1)) break;
+    ItemRow my = rows.at(I, it);
+    for (uint64_t b = b0; b < b1; ++b) {
+      const uint64_t local = (block0 + b) * kWarp + lane;
+      const bool act[1] = {local < L.path_count};
+      const uint64_t pth[1] = {L.path_begin + local};
+      float x[1], comp[1], g[1][5];
+      const SegGlobal seg{gseg, (long long)blockIdx.x * bd + tid, A.ckpt_every, (long long)ck_stride};
+      if (tab)
+        path_adjoint_ppt<1, SegGlobal, true, QEM, true>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
+                                                        seg, x, comp, g, L.qm, tab);
+      else
+        path_adjoint_ppt<1, SegGlobal, true, QEM, false>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
+                                                         seg, x, comp, g, L.qm);
+      const float S[1] = {terminal_spot(L.S0, x[0], comp[0])};
+      if (TILE == 1) {
+        for (int a = 0; a < kAdjAcc; ++a) {
+          const float t = warp_sum(act[0] ? adj_term(a, put, S[0], ks[0].K, g[0], A.invS0, A.T) : 0.0f);
+          if (lane == 0) my.add(a, t);
+        }
+      } else {
+        for (int t0 = 0; t0 < L.nk_pad; t0 += 32) {
+          float t[kAdjAcc];
+          strike_tile_terms<1>(put, ks[t0 + lane].K, S, act, g, t);
+#pragma unroll
+          for (int a = 0; a < kAdjAcc; ++a) my.add(a * L.nk_pad + t0 + lane, t[a]);
+        }
+      }
+      my.first = false;
     }
   }
-  if (threadIdx.x == 0) *ticket = 0u;
+  __syncthreads();
+  sum_item_rows(rows, I, nb);
+  __syncthreads();
+  if (!sum_block_rows(rows.acc, rows.row, partials, ticket, s_flag)) return;
+  // (a tile's third sum holds the weights w: the S0 column is w / S0)
+  write_adjoint(L, A, strikes, rows.acc, TILE == 1 ? 1.0 : (double)A.invS0, out);
 }
 
 // Per-path output: x_T and g = d x_T / d(v0, kappa, theta, sigma, rho).
@@ -265,43 +336,63 @@ __global__ void __launch_bounds__(128) heston_paths_adjoint_kernel(const __grid_
   for (int j = 0; j < 5; ++j) grad[i * 5 + j] = g[0][j];
 }
 
-// The grid of the per-strike kernel variant (resident blocks, at most what the
-// paths need) and its dynamic shared memory.
-template <int TILE, bool RACC, bool GSEG, bool QEM>
-cudaError_t adjoint_grid_t(const PathLaunch& L, const AdjConst& A, int num_sms, uint64_t* grid, size_t* smem) {
-  constexpr int PPT = SIMR_ADJ_PPT;
-  const int tpb = 128, warps = tpb / kWarp;
-  *smem = adjoint_smem_bytes_t(L, A, tpb, PPT, RACC, GSEG);
-  auto kern = heston_adjoint_kernel<TILE, PPT, RACC, GSEG, QEM>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tpb, *smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const uint64_t batches = (L.path_count + (uint64_t)kWarp * PPT - 1) / ((uint64_t)kWarp * PPT);
-  uint64_t g = (uint64_t)num_sms * per_sm;
-  const uint64_t need = (batches + warps - 1) / warps;
-  if (g > need) g = need;
-  *grid = g < 1 ? 1 : g;
-  return cudaSuccess;
-}
-
-template <int TILE, bool RACC, bool GSEG, bool QEM>
+template <int TILE, bool RACC, bool QEM>
 cudaError_t launch_adjoint_t(const PathLaunch& L, const AdjConst& A, const double* strikes, const AdjOutputs& out,
                              const Scratch& s, int num_sms, cudaStream_t stream) {
   constexpr int PPT = SIMR_ADJ_PPT;
-  const int tpb = 128;
+  const int tpb = 128, warps = tpb / kWarp;
   const size_t row = (size_t)kAdjAcc * L.nk_pad;
-  uint64_t grid = 0;
-  size_t smem = 0;
-  cudaError_t e = adjoint_grid_t<TILE, RACC, GSEG, QEM>(L, A, num_sms, &grid, &smem);
+  const size_t smem = adjoint_smem_bytes_t(L, A, tpb, PPT, RACC);
+  auto kern = heston_adjoint_kernel<TILE, PPT, RACC, QEM>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  if ((size_t)grid * row > s.partial_doubles) return cudaErrorMemoryAllocation;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tpb, smem);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const uint64_t batches = (L.path_count + (uint64_t)kWarp * PPT - 1) / ((uint64_t)kWarp * PPT);
+  const uint64_t need = (batches + warps - 1) / warps;
+  const uint64_t grid = std::min<uint64_t>((uint64_t)num_sms * per_sm, need);
+  if ((size_t)(grid + kRowGroups) * row > s.partial_doubles) return cudaErrorMemoryAllocation;
   if ((size_t)grid * tpb * adjoint_ckpt_floats(A, PPT) > s.ckpt_floats) return cudaErrorMemoryAllocation;
-  if (GSEG && (size_t)grid * tpb * adjoint_seg_floats(A, PPT) > s.gseg_floats) return cudaErrorMemoryAllocation;
-  heston_adjoint_kernel<TILE, PPT, RACC, GSEG, QEM>
-      <<<(unsigned)grid, tpb, smem, stream>>>(L, A, strikes, out, s.partials, s.ticket, s.ckpt, s.gseg);
+  kern<<<(unsigned)grid, tpb, smem, stream>>>(L, A, strikes, out, s.partials, s.ticket, s.ckpt);
+  return cudaGetLastError();
+}
+
+// The launch shape of the global-segment kernel: items, table, shared memory.
+struct SegShape {
+  ItemPlan I;
+  uint64_t grid;
+  int pair_table;
+  size_t smem;
+};
+SegShape seg_shape(const PathLaunch& L, int num_sms, bool qem) {
+  SegShape h;
+  h.pair_table = pair_table_entries(L);
+  const size_t row = (size_t)kAdjAcc * L.nk_pad;
+  const size_t head = L.nk_pad * sizeof(StrikeConst) + 16 + h.pair_table * sizeof(uint4);
+  const uint64_t batches = (L.path_count + kWarp - 1) / kWarp;
+  h.grid = std::max<uint64_t>(1, std::min<uint64_t>(num_sms, batches));
+  h.I = make_item_plan(batches, h.grid, qem ? SIMR_ADJ_QEM_WARPS : SIMR_ADJ_WARPS, row, kItemBytes - head);
+  h.smem = head + item_rows_bytes(h.I, row);
+  return h;
+}
+
+template <int TILE, bool QEM>
+cudaError_t launch_adjoint_seg(const PathLaunch& L0, const AdjConst& A, const double* strikes, const AdjOutputs& out,
+                               const Scratch& s, int num_sms, cudaStream_t stream) {
+  const SegShape h = seg_shape(L0, num_sms, QEM);
+  PathLaunch L = L0;
+  L.pair_table = h.pair_table;
+  const int tpb = kWarp * h.I.warps;
+  const size_t row = (size_t)kAdjAcc * L.nk_pad;
+  auto kern = heston_adjoint_seg_kernel<TILE, QEM>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem);
+  if (e != cudaSuccess) return e;
+  if ((size_t)(h.grid + kRowGroups) * row > s.partial_doubles) return cudaErrorMemoryAllocation;
+  if ((size_t)h.grid * tpb * adjoint_ckpt_floats(A, 1) > s.ckpt_floats) return cudaErrorMemoryAllocation;
+  if ((size_t)h.grid * tpb * adjoint_seg_floats(A, 1) > s.gseg_floats) return cudaErrorMemoryAllocation;
+  kern<<<(unsigned)h.grid, tpb, h.smem, stream>>>(L, A, h.I, strikes, out, s.partials, s.ticket, s.ckpt, s.gseg);
   return cudaGetLastError();
 }
 
@@ -317,27 +408,27 @@ template <bool QEM>
 cudaError_t launch_adjoint_s(const PathLaunch& L, const AdjConst& A, const double* strikes, const AdjOutputs& out,
                              const Scratch& s, int num_sms, cudaStream_t stream) {
   if (adjoint_gseg(L, A)) {
-    if (L.nk_pad == 1) return launch_adjoint_t<1, false, true, QEM>(L, A, strikes, out, s, num_sms, stream);
-    if (L.nk_pad == 32) return launch_adjoint_t<32, true, true, QEM>(L, A, strikes, out, s, num_sms, stream);
-    return launch_adjoint_t<32, false, true, QEM>(L, A, strikes, out, s, num_sms, stream);
+    return L.nk_pad == 1 ? launch_adjoint_seg<1, QEM>(L, A, strikes, out, s, num_sms, stream)
+                         : launch_adjoint_seg<32, QEM>(L, A, strikes, out, s, num_sms, stream);
   }
-  if (L.nk_pad == 1) return launch_adjoint_t<1, false, false, QEM>(L, A, strikes, out, s, num_sms, stream);
-  if (L.nk_pad == 32) return launch_adjoint_t<32, true, false, QEM>(L, A, strikes, out, s, num_sms, stream);
-  return launch_adjoint_t<32, false, false, QEM>(L, A, strikes, out, s, num_sms, stream);
+  if (L.nk_pad == 1) return launch_adjoint_t<1, false, QEM>(L, A, strikes, out, s, num_sms, stream);
+  if (L.nk_pad == 32) return launch_adjoint_t<32, true, QEM>(L, A, strikes, out, s, num_sms, stream);
+  return launch_adjoint_t<32, false, QEM>(L, A, strikes, out, s, num_sms, stream);
 }
 
 }  // namespace
 
 size_t adjoint_scratch_doubles(const PathLaunch& L, int num_sms) {
-  return (size_t)num_sms * 16 * kAdjAcc * (size_t)L.nk_pad;  // at most 16 resident blocks of 128 threads per SM
+  // at most 16 resident blocks of 128 threads per SM
+  return ((size_t)num_sms * 16 + kRowGroups) * kAdjAcc * (size_t)L.nk_pad;
 }
 
 cudaError_t adjoint_max_ckpt_every(const PathLaunch& L, int steps_cap, int* k_max) {
   // the kernel variant launch_adjoint picks for this strike count
   const bool racc = L.nk_pad == 32;
-  const void* kern = L.nk_pad == 1 ? (const void*)heston_adjoint_kernel<1, SIMR_ADJ_PPT, false, false, false>
-                     : racc      ? (const void*)heston_adjoint_kernel<32, SIMR_ADJ_PPT, true, false, false>
-                                 : (const void*)heston_adjoint_kernel<32, SIMR_ADJ_PPT, false, false, false>;
+  const void* kern = L.nk_pad == 1 ? (const void*)heston_adjoint_kernel<1, SIMR_ADJ_PPT, false, false>
+                     : racc      ? (const void*)heston_adjoint_kernel<32, SIMR_ADJ_PPT, true, false>
+                                 : (const void*)heston_adjoint_kernel<32, SIMR_ADJ_PPT, false, false>;
   auto blocks = [&](int k, int* n) -> cudaError_t {
     AdjConst A{};
     A.ckpt_every = k;
@@ -371,20 +462,9 @@ size_t adjoint_smem_bytes(const PathLaunch& L, const AdjConst& A) {
 cudaError_t adjoint_gseg_floats(const PathLaunch& L, const AdjConst& A, int num_sms, size_t* floats) {
   *floats = 0;
   if (!adjoint_gseg(L, A)) return cudaSuccess;
-  uint64_t grid = 0;
-  size_t smem = 0;
-  cudaError_t e = L.nk_pad == 1    ? adjoint_grid_t<1, false, true, false>(L, A, num_sms, &grid, &smem)
-                  : L.nk_pad == 32 ? adjoint_grid_t<32, true, true, false>(L, A, num_sms, &grid, &smem)
-                                   : adjoint_grid_t<32, false, true, false>(L, A, num_sms, &grid, &smem);
-  if (e == cudaSuccess && L.scheme == 1) {  // the QE-M kernel's occupancy may differ: take the larger grid
-    uint64_t grid_q = 0;
-    e = L.nk_pad == 1    ? adjoint_grid_t<1, false, true, true>(L, A, num_sms, &grid_q, &smem)
-        : L.nk_pad == 32 ? adjoint_grid_t<32, true, true, true>(L, A, num_sms, &grid_q, &smem)
-                         : adjoint_grid_t<32, false, true, true>(L, A, num_sms, &grid_q, &smem);
-    if (grid_q > grid) grid = grid_q;
-  }
-  if (e == cudaSuccess) *floats = (size_t)grid * 128 * adjoint_seg_floats(A, SIMR_ADJ_PPT);
-  return e;
+  const SegShape h = seg_shape(L, num_sms, L.scheme == 1);
+  *floats = (size_t)h.grid * kWarp * h.I.warps * adjoint_seg_floats(A, 1);
+  return cudaSuccess;
 }
 
 size_t adjoint_ckpt_scratch_floats(const AdjConst& A, int num_sms) {

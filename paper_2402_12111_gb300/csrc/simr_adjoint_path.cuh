@@ -469,13 +469,56 @@ __device__ __forceinline__ float branch_draw(const ScenConst& c, float v, float 
   return qe_t(m * m, s2h) > kQuadT ? zv : one_minus_u(xv);
 }
 
-// The stored data of one step (recompute pass): (state, branch draw) as one
-// pair and Z_X, from the step's centred variance uniform and its two normals.
-__device__ __forceinline__ void keep_step(const ScenConst& c, float xv_v, float zv, float zx, float2* bvd, float* bz,
+// One step of the recompute pass: the stored data -- (state, branch draw) as one
+// pair and Z_X -- and the next state, from the step's centred variance uniform and
+// its two normals.
+__device__ __forceinline__ void keep_step(const ScenConst& c, float xv, float zv, float zx, float2* bvd, float* bz,
                                           float& v) {
-  *bvd = make_float2(v, branch_draw(c, v, xv_v, zv));
+  *bvd = make_float2(v, branch_draw(c, v, xv, zv));
   *bz = zx;
-  v = qe_only(c, v, xv_v, zv);
+  v = qe_only(c, v, xv, zv);
+}
+
+// The draws of a step pair: 2 U_V - 1, Z_V and Z_X, lane x the even step's.
+struct PairDraw {
+  float2 xv, zv, zx;
+};
+
+__device__ __forceinline__ bool pair_draw_try(const uint4& w, PairDraw& d, float2& xx, float2& wcv, float2& wcx) {
+  d.xv = centered_uniform2(w.x, w.z);
+  xx = centered_uniform2(w.y, w.w);
+  const bool a = norminv_try2(d.xv, wcv, d.zv);
+  return norminv_try2(xx, wcx, d.zx) && a;
+}
+__device__ __forceinline__ void pair_draw_fix(PairDraw& d, float2 xx, float2 wcv, float2 wcx) {
+  norminv_fix2(d.xv, wcv, d.zv);
+  norminv_fix2(xx, wcx, d.zx);
+}
+
+// keep_step of the even step of a pair and the draws of the next pair, from its
+// words: independent of each other, and what leaves the common path (a tail
+// normal, the exponential branch) is redone behind one test.
+__device__ __forceinline__ void keep_step_pipe(const ScenConst& c, const PairDraw& d, const uint4& wn, PairDraw& dn,
+                                               float2* bvd, float* bz, float& v) {
+  const float m = fmaf(v, c.E, c.thE);
+  const float s2h = fmaf(v, c.h1, c.h2);
+  const float m2 = __fmul_rn(m, m);
+  const float t = qe_t(m2, s2h);
+  float vn, dl, dr = d.zv.x;
+  qe_quad_branch(m, t, d.zv.x, vn, dl);
+  const bool quad = t > kQuadT;
+  float2 xx, wcv, wcx;
+  const bool central = pair_draw_try(wn, dn, xx, wcv, wcx);
+  if (!(quad && central)) {
+    pair_draw_fix(dn, xx, wcv, wcx);
+    if (!quad) {
+      dr = one_minus_u(d.xv.x);
+      qe_exp_branch(m, s2h, m2, d.xv.x, vn, dl);
+    }
+  }
+  *bvd = make_float2(v, dr);
+  *bz = d.zx.x;
+  v = vn;
 }
 
 // A thread's column of a segment buffer of `stride` columns (8-byte aligned):
@@ -531,9 +574,9 @@ __device__ __forceinline__ void adjoint_map(const AdjConst& A, const AdjSums& a,
 // thread's segment column S (at least k rows) -- then the steps are
 // differentiated backwards.  x_T (with its Kahan remainder) is summed on the
 // way; g = d x_T / d(v0, kappa, theta, sigma, rho).
-template <typename Seg, bool PAIRED, bool QEM = false>
+template <typename Seg, bool PAIRED, bool QEM, bool TAB>
 __device__ __forceinline__ void path_sweep(const ScenConst& c, const AdjConst& A, uint32_t N, uint32_t option,
-                                           const uint32_t (&rk)[10][2], const PhiloxLane& pl,
+                                           const uint32_t (&rk)[10][2], const uint4* tab, const PhiloxLane& pl0,
                                            const float* ck, int cstride, float v_last, const Seg& S,
                                            float& x_out, float& comp_out, float (&g)[5], const QemConst& qm) {
   using I = decltype(S.stride());
@@ -541,6 +584,7 @@ __device__ __forceinline__ void path_sweep(const ScenConst& c, const AdjConst& A
   const float c1 = c.h1 + c.h1;  // s^2 = v c1 + c2
   const uint32_t k = (uint32_t)A.ckpt_every;
   const int n_seg = A.n_seg;
+  const PhiloxLane pl[1] = {pl0};
   AdjSums as = AdjSums{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
   float2* s01 = S.pairs();
   float* s2 = S.zx();
@@ -554,13 +598,19 @@ __device__ __forceinline__ void path_sweep(const ScenConst& c, const AdjConst& A
     // this thread's column, by pointers stepped two rows per pair (n0 is even)
     float2* wp = s01;
     float* wz = s2;
+    PairDraw d, dn;
+    uint4 w[1];
+    philox_draws<TAB, 1>(tab, n0 / 2, option, rk, pl, w);
+    {
+      float2 xx, wcv, wcx;
+      if (!pair_draw_try(w[0], d, xx, wcv, wcx)) pair_draw_fix(d, xx, wcv, wcx);
+    }
+#pragma unroll 1
     for (uint32_t p = n0 / 2; 2 * p < n1; ++p, wp += 2 * bd, wz += 2 * bd) {
-      const uint4 w = philox_draw(pl, philox_ctr(p, option, rk), rk);
-      const float2 xv = centered_uniform2(w.x, w.z);
-      const float2 zv = norminv_centered2(xv);  // the pair's normals two at a time
-      const float2 zx = norminv_centered2(centered_uniform2(w.y, w.w));
-      keep_step(c, xv.x, zv.x, zx.x, wp, wz, vv);
-      if (2 * p + 1 < n1) keep_step(c, xv.y, zv.y, zx.y, wp + bd, wz + bd, vv);
+      philox_draws<TAB, 1>(tab, p + 1, option, rk, pl, w);  // (the pair past the segment is drawn and not used)
+      keep_step_pipe(c, d, w[0], dn, wp, wz, vv);
+      if (2 * p + 1 < n1) keep_step(c, d.xv.y, d.zv.y, d.zx.y, wp + bd, wz + bd, vv);
+      d = dn;
     }
     float vnext = vv;  // v_{n1}
     // the reverse steps read row i by pointers rp, rz stepped down from the top row
@@ -671,12 +721,12 @@ __device__ __forceinline__ void path_sweep(const ScenConst& c, const AdjConst& A
 // Checkpoint (slot, path j) of this thread at ck[(slot * PPT + j) * ck_stride]
 // (n_seg - 1 slots; shared or global memory); S is this thread's segment column
 // (shared or global memory, at least k rows).
-template <int PPT, typename Seg, bool PAIRED = true, bool QEM = false>
+template <int PPT, typename Seg, bool PAIRED = true, bool QEM = false, bool TAB = false>
 __device__ __forceinline__ void path_adjoint_ppt(const ScenConst& c, const AdjConst& A, uint32_t N, uint32_t option,
                                                  const uint32_t (&rk)[10][2], const uint64_t (&path)[PPT], float* ck,
                                                  int ck_stride, const Seg& S, float (&x_out)[PPT],
                                                  float (&comp_out)[PPT], float (&g)[PPT][5],
-                                                 const QemConst& qm = QemConst{}) {
+                                                 const QemConst& qm = QemConst{}, const uint4* tab = nullptr) {
   static_assert(PPT == 1 || PPT == 2, "one or two paths per thread");
   const uint32_t k = (uint32_t)A.ckpt_every;
   const int n_seg = A.n_seg;
@@ -694,8 +744,7 @@ __device__ __forceinline__ void path_adjoint_ppt(const ScenConst& c, const AdjCo
     const uint32_t p0 = (uint32_t)sg * (k / 2);
     for (uint32_t p = p0; p < p0 + k / 2; ++p) {
       uint4 w[PPT];
-#pragma unroll
-      for (int j = 0; j < PPT; ++j) w[j] = philox_draw(pl[j], philox_ctr(p, option, rk), rk);
+      philox_draws<TAB, PPT>(tab, p, option, rk, pl, w);
       if constexpr (PPT == 2) {
         const float2 xa = centered_uniform2(w[0].x, w[1].x), xb = centered_uniform2(w[0].z, w[1].z);
         const float2 za = norminv_centered2(xa);
@@ -716,7 +765,7 @@ __device__ __forceinline__ void path_adjoint_ppt(const ScenConst& c, const AdjCo
   }
 #pragma unroll
   for (int j = 0; j < PPT; ++j)
-    path_sweep<Seg, PAIRED, QEM>(c, A, N, option, rk, pl[j], ck + j * ck_stride, PPT * ck_stride, v[j], S,
+    path_sweep<Seg, PAIRED, QEM, TAB>(c, A, N, option, rk, tab, pl[j], ck + j * ck_stride, PPT * ck_stride, v[j], S,
                                  x_out[j], comp_out[j], g[j], qm);
 }
 

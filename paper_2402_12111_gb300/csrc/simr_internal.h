@@ -128,6 +128,7 @@ struct BatchLaunch {
   int32_t seg_rows;   // adjoint: rows of each segment array (max over options of ckpt_every)
   float* gseg;        // adjoint with one segment per path: [3 seg_rows][grid threads] in global memory, else null
   size_t gseg_floats;  // its capacity
+  int32_t tab_rows;    // entries of each warp's step-pair counter table, 0: none (shared segments have none)
   int32_t tpb, ppt, unroll;  // the kernel's shape (batch_variant)
   int32_t qem;               // 1: the options' log-spot steps under QE-M
 };
@@ -164,6 +165,9 @@ inline size_t item_rows_bytes(const ItemPlan& I, size_t row) {
 }
 // Dynamic shared memory a path kernel's block may take for them.
 constexpr size_t kItemBytes = 208 * 1024;
+// Entries of the shared-memory table of step-pair counters for L's paths and steps.
+struct PathLaunch;
+int pair_table_entries(const PathLaunch& L);
 // Groups of blocks of the two-level sum over blocks: words 1 .. kRowGroups of the
 // ticket block count their arrivals.
 constexpr int kRowGroups = 15;

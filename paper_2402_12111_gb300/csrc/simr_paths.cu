@@ -467,16 +467,6 @@ __global__ void __launch_bounds__(256) heston_terminal_kernel(const __grid_const
   if (v_T) v_T[i] = v[0][0];
 }
 
-// Entries of the shared-memory table of step-pair counters: one per pair and one
-// past the last, which a pipelined loop reads; none where the paths cross a
-// multiple of 2^32 (their high words differ), or past 32 KB (4,092 steps), which
-// the items' rows need more.
-int pair_table_entries(const PathLaunch& L) {
-  const uint64_t n = (uint64_t)L.steps / 2 + 2;
-  const bool one_high_word = (L.path_begin >> 32) == ((L.path_begin + L.path_count - 1) >> 32);
-  return one_high_word && n <= 2048 ? (int)n : 0;
-}
-
 template <int NS, int NV, int TILE, bool DYN, bool QEM = false,
           int PPT = (NS == 1 ? SIMR_PRICE_PPT : SIMR_FD_PPT)>
 cudaError_t launch_t(const PathLaunch& L0, const double* strikes, const PathOutputs& out, const Scratch& s,
@@ -501,6 +491,16 @@ cudaError_t launch_t(const PathLaunch& L0, const double* strikes, const PathOutp
 
 }  // namespace
 
+// Entries of the shared-memory table of step-pair counters: one per pair and one
+// past the last, which a pipelined loop reads; none where the paths cross a
+// multiple of 2^32 (their high words differ), or past 32 KB (4,092 steps), which
+// the items' rows need more.
+int pair_table_entries(const PathLaunch& L) {
+  const uint64_t n = (uint64_t)L.steps / 2 + 2;
+  const bool one_high_word = (L.path_begin >> 32) == ((L.path_begin + L.path_count - 1) >> 32);
+  return one_high_word && n <= 2048 ? (int)n : 0;
+}
+
 ItemPlan make_item_plan(uint64_t batches, uint64_t grid, int max_warps, size_t row, size_t bytes) {
   ItemPlan I{};
   I.batches = batches;
@@ -510,7 +510,7 @@ ItemPlan make_item_plan(uint64_t batches, uint64_t grid, int max_warps, size_t r
   // few batches a warp: as many warps as make the rounds even (31 batches on 28
   // warps: two rounds of 16, not 28 and 3)
   const uint64_t rounds = (most + w - 1) / w;
-  if (rounds <= 4) w = (most + rounds - 1) / rounds;
+  if (rounds == 2) w = (most + rounds - 1) / rounds;
   I.warps = (int)w;
   bytes -= std::max<size_t>(row, 32 * w) * 8 + 8;
   // the fewest levels after which the rest, batch by batch in FP32 rows, fits; if

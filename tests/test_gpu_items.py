@@ -101,3 +101,63 @@ def test_step_counts_match_the_per_path_simulation(simr, steps, scheme, model):
     S = m["S0"] * torch.exp(x.double())
     ref = np.exp(-m["r"] * m["T"]) * torch.clamp(S[None] - K[:, None], min=0.0).mean(1)
     assert torch.all((p - ref).abs() <= 1e-6 * S.mean()), (p, ref)
+
+
+@pytest.mark.parametrize("scheme", ["qe", "qem"])
+@pytest.mark.parametrize("paths,n_strikes", [(1, 1), (31, 32), (32 * SMS + 1, 1), (32 * SMS * 24 + 5, 33),
+                                             (32 * SMS * 150 + 17, 32), (32 * SMS * 40 + 3, 256)])
+def test_adjoint_with_a_global_segment_equals_shared_segments(simr, paths, n_strikes, scheme):
+    # the two kernels form the same FP32 sums of 32 paths (one hands out items, one
+    # strides); an odd step count and one segment past the even one
+    K = torch.linspace(80.0, 120.0, n_strikes, dtype=torch.float64, device="cuda") if n_strikes > 1 else \
+        torch.tensor([100.0], dtype=torch.float64, device="cuda")
+    m = dict(workloads.BASE_MODEL, sigma=0.6)
+    with simr.scheme(scheme):
+        a = simr.greeks_adjoint(m, K, True, 171, paths, 3)  # 171 steps: one segment, too long for shared memory
+        b = simr.greeks_adjoint(m, K, True, 171, paths, 3, ckpt_every=16)
+    for x, y in zip(a, b):
+        scale = y.abs().amax(dim=0, keepdim=True).clamp_min(1e-300)
+        assert torch.all((x - y).abs() <= 1e-11 * scale), float(((x - y).abs() / scale).max())
+
+
+@pytest.mark.parametrize("scheme", ["qe", "qem"])
+@pytest.mark.parametrize("n_assets", [1, 2, 3, 4, 5, 8, 9, 16])
+@pytest.mark.parametrize("steps,paths", [(3, 32 * SMS * 17 + 9), (600, 97)])  # 600 steps x 16 assets: no counter table
+def test_basket_of_one_weight_is_the_single_asset_price(simr, n_assets, steps, paths, scheme):
+    # uncorrelated assets with the last one's weight 1 and the rest 0: the last
+    # asset's own European price on the paths of its option index.  FP32 sums of 32
+    # paths against 64: 6 roundings of 2^-24 each, 4e-7
+    m = workloads.random_models(n_assets, 5)
+    for q in m:
+        q["T"], q["r"] = 1.0, 0.03
+    w = np.zeros(n_assets)
+    w[-1] = 1.0
+    K = torch.linspace(80.0, 120.0, 33, dtype=torch.float64, device="cuda")
+    with simr.scheme(scheme):
+        p, _ = simr.basket_price(m, np.eye(n_assets), w, K, False, steps, paths, 7)
+        q, _ = simr.price(m[-1], K, False, steps, paths, 7, option_index=n_assets - 1)
+    torch.testing.assert_close(p, q, rtol=4e-7, atol=4e-7)
+
+
+@pytest.mark.parametrize("paths", [2, 63, 65, 64 * SMS * 24 + 1, 64 * SMS * 100 + 31])
+@pytest.mark.parametrize("steps", [1, 7, 4095])
+def test_one_exercise_date_is_the_european_price(simr, steps, paths):
+    # the Longstaff-Schwartz path kernel against the pricing kernel on the same paths
+    # (FP32 sums grouped differently: 4e-7 as above, of a mean payoff above 1)
+    if steps == 4095 and paths > 70:
+        pytest.skip("long paths at small counts only")
+    m = dict(workloads.BASE_MODEL)
+    p = simr.lsm_price(m, 110.0, True, steps, steps, paths, 5)[0]
+    q, _ = simr.price(m, torch.tensor([110.0], dtype=torch.float64, device="cuda"), True, steps, paths, 5)
+    torch.testing.assert_close(p, q, rtol=4e-7, atol=4e-7)
+
+
+def test_book_rows_beyond_one_per_lane(simr):
+    # more work items than the reducing warp has lanes, and one path
+    book = [dict(model=dict(workloads.BASE_MODEL), K=100.0, is_put=False, steps=3, paths=n) for n in (1, 64 * 33 + 1, 100003)]
+    p, se, _ = simr.batch(book, seed=4, autotune=False)
+    for i, o in enumerate(book):
+        q, sq = simr.price(o["model"], torch.tensor([100.0], dtype=torch.float64, device="cuda"), False, 3, o["paths"], 4,
+                           option_index=i)
+        torch.testing.assert_close(p[i:i + 1], q, rtol=1e-12, atol=1e-12)
+        torch.testing.assert_close(se[i:i + 1], sq, rtol=1e-9, atol=1e-12)
