@@ -1250,16 +1250,21 @@ int simr_batch_submit(simr_ctx* ctx, const simr_option* opts, int n_opts, uint64
   // kAdjAutoGsegFloats; else checkpoints and segments in shared memory
   bool one_segment = false;
   size_t gseg_floats = 0;
-  if (adjoint) {
-    uint32_t max_steps = 0;
-    for (int i = 0; i < n_opts; ++i) max_steps = std::max(max_steps, opts[i].steps);
-    if (max_steps >= 1 && max_steps <= 1024) {
-      size_t threads = 0;
-      cudaError_t eg = batch_gseg_threads(ctx->num_sms, &threads);
-      if (eg != cudaSuccess) return cuda_fail(eg, "sizing the book's segment buffers");
-      gseg_floats = (size_t)3 * (max_steps + (max_steps & 1u)) * threads;
-      one_segment = gseg_floats <= kAdjAutoGsegFloats;
-    }
+  uint32_t max_steps = 0;
+  uint64_t max_paths = 0;
+  for (int i = 0; i < n_opts; ++i) {
+    max_steps = std::max(max_steps, opts[i].steps);
+    max_paths = std::max(max_paths, opts[i].paths);
+  }
+  // each warp's table of its option's step-pair counters: where a block's tables
+  // stay small (66 KB at 1,024 steps) and all paths have the high counter word 0
+  const bool tables = max_steps >= 1 && max_steps <= 1024 && max_paths <= (1ull << 32);
+  if (adjoint && tables) {
+    size_t threads = 0;
+    cudaError_t eg = batch_gseg_threads(ctx->num_sms, &threads);
+    if (eg != cudaSuccess) return cuda_fail(eg, "sizing the book's segment buffers");
+    gseg_floats = (size_t)3 * (max_steps + (max_steps & 1u)) * threads;
+    one_segment = gseg_floats <= kAdjAutoGsegFloats;
   }
   int ckpt_rows = 0, seg_rows = 0;
   if ((rc = build_batch_options(opts, n_opts, adjoint, qem, &bo, one_segment, &order, &ckpt_rows, &seg_rows)))
@@ -1275,6 +1280,7 @@ int simr_batch_submit(simr_ctx* ctx, const simr_option* opts, int n_opts, uint64
   B.ckpt_rows = ckpt_rows;
   B.seg_rows = seg_rows;
   B.gseg = one_segment ? ctx->gseg : nullptr;
+  B.tab_rows = tables && (one_segment || !adjoint) ? (int32_t)(max_steps / 2 + 2) : 0;
   B.qem = qem ? 1 : 0;
   const int nacc = adjoint ? 9 : 2;
   OutStage o;

@@ -28,27 +28,34 @@ namespace {
 // together in packed FP32, or 1 at a time -- each lane then adds its two paths'
 // terms in the same order, so both give the same sums bit for bit); U, the
 // unrolling of the step-pair loop.
-// Adjoint books ask the register allocator for 640 resident threads per SM (5
-// blocks of 128: at most 102 registers), which it would otherwise trade for
-// registers it does not need (measured on the 1,024-option book with paired
-// reverse steps: 311 ms, against 317 at 768 threads and 393 with no bound).
+// Resident threads per SM asked of the register allocator: adjoint books 768 (80
+// registers; QE-M 8.7 ms against 8.9 at 640 threads on 16 options, QE the same),
+// price books with the pipelined pair of paths 512 (7.5 -> 6.6 ms for 64 options,
+// QE-M 5.35 -> 3.4 ms for 16; 640 and 768 within 3%).
 #ifndef SIMR_BOOK_PAIRED
 #define SIMR_BOOK_PAIRED true  // reverse steps in pairs (one at a time: 351 ms against 311 for the book)
 #endif
 #ifndef SIMR_BOOK_ADJ_THREADS
-#define SIMR_BOOK_ADJ_THREADS 640
+#define SIMR_BOOK_ADJ_THREADS 768
+#endif
+#ifndef SIMR_BOOK_PRICE_THREADS
+#define SIMR_BOOK_PRICE_THREADS 512
 #endif
 // QEM: the options' log-spot steps under QE-M (their QemConst); price books
 // then run two paths per thread, unrolled once (two shapes: the block size).
 template <bool ADJ, bool GSEG, int TPB, int PPT, int U, bool QEM>
-__global__ void __launch_bounds__(TPB, ADJ ? SIMR_BOOK_ADJ_THREADS / TPB : 1) heston_batch_kernel(const __grid_constant__ BatchLaunch B,
+__global__ void __launch_bounds__(TPB, ADJ ? SIMR_BOOK_ADJ_THREADS / TPB : PPT == 2 && U == 1 ? SIMR_BOOK_PRICE_THREADS / TPB : 1) heston_batch_kernel(const __grid_constant__ BatchLaunch B,
                                                            const BatchOption* __restrict__ opts,
                                                            const BatchItem* __restrict__ items,
                                                            unsigned int* __restrict__ counter,
                                                            double* __restrict__ partials) {
   extern __shared__ __align__(16) float smem_f[];
   constexpr int NACC = ADJ ? kAdjAcc : 2;
+  constexpr bool TABLE = ADJ ? GSEG : PPT == 2 && U == 1;  // the shapes that read the table
   const int lane = threadIdx.x & 31, tid = threadIdx.x, bd = blockDim.x;
+  // this warp's table of its option's step-pair counters (no table: tab_rows 0)
+  uint4* tab = reinterpret_cast<uint4*>(smem_f) + (size_t)(tid >> 5) * B.tab_rows;
+  uint32_t tab_option = 0xffffffffu;
   while (true) {
     unsigned int it = 0;
     if (lane == 0) it = atomicAdd(counter, 1u);
@@ -60,6 +67,12 @@ __global__ void __launch_bounds__(TPB, ADJ ? SIMR_BOOK_ADJ_THREADS / TPB : 1) he
     const float K = O.K, S0 = O.S0;
     const bool put = O.is_put != 0;
     const uint32_t steps = O.steps, oidx = O.option_index;
+    if (TABLE && B.tab_rows && tab_option != I.option) {
+      __syncwarp();
+      for (uint32_t p = lane; p < steps / 2 + 2; p += 32) tab[p] = philox_pair_entry(p, oidx, 0u, B.rk);
+      __syncwarp();
+      tab_option = I.option;
+    }
     double acc[NACC];
 #pragma unroll
     for (int a = 0; a < NACC; ++a) acc[a] = 0.0;
@@ -77,10 +90,10 @@ __global__ void __launch_bounds__(TPB, ADJ ? SIMR_BOOK_ADJ_THREADS / TPB : 1) he
         // arrays of seg_rows rows (the largest over the book), so threads on
         // options with different checkpoint intervals never overlap
         if constexpr (GSEG)  // one segment: no checkpoints are read or written
-          path_adjoint_ppt<1, SegGlobal, SIMR_BOOK_PAIRED, QEM>(
+          path_adjoint_ppt<1, SegGlobal, SIMR_BOOK_PAIRED, QEM, true>(
               c, O.A, steps, oidx, B.rk, pth, B.gseg, 0,
               SegGlobal{B.gseg, (long long)blockIdx.x * bd + tid, B.seg_rows, (long long)gridDim.x * bd}, x, comp,
-              g, O.qm);
+              g, O.qm, tab);
         else
           path_adjoint_ppt<1, SegShared, SIMR_BOOK_PAIRED, QEM>(c, O.A, steps, oidx, B.rk, pth, smem_f + tid, bd,
                                                                 SegShared{smem_f + B.ckpt_rows * bd, B.seg_rows},
@@ -92,9 +105,14 @@ __global__ void __launch_bounds__(TPB, ADJ ? SIMR_BOOK_ADJ_THREADS / TPB : 1) he
         terms[0] = terms[1] = 0.0f;
         float xs[2], cs[2];
         if constexpr (PPT == 2) {
-          float2 x2, comp2;
-          simulate_two<U, QEM>(c, steps, oidx, B.rk, I.path_begin + b + lane, I.path_begin + b + 32 + lane, x2,
-                               comp2, O.qm);
+          float2 v2, x2, comp2;
+          const uint64_t p0 = I.path_begin + b + lane, p1 = p0 + 32;
+          if constexpr (U > 1)
+            simulate_two<U, QEM>(c, steps, oidx, B.rk, p0, p1, x2, comp2, O.qm);
+          else if (B.tab_rows)
+            simulate_two_pipe<QEM, true>(c, steps, oidx, B.rk, tab, p0, p1, v2, x2, comp2, O.qm, [](uint32_t) {});
+          else
+            simulate_two_pipe<QEM, false>(c, steps, oidx, B.rk, tab, p0, p1, v2, x2, comp2, O.qm, [](uint32_t) {});
           xs[0] = x2.x;
           xs[1] = x2.y;
           cs[0] = comp2.x;
@@ -123,16 +141,30 @@ __global__ void __launch_bounds__(TPB, ADJ ? SIMR_BOOK_ADJ_THREADS / TPB : 1) he
   }
 }
 
-// One thread per option: sum its items' rows in item order, normalise.
+// One warp per option: lane l sums the rows of its items l, l + 32, ... in order, a
+// butterfly the lanes, and lane 0 normalises.  (One thread per option added up to
+// 1,024 rows one after another: 5 options of 25,000 paths, 391 rows each, spent
+// 200 of a submission's 300 us here.)
 __global__ void batch_reduce_kernel(const BatchOption* __restrict__ opts, uint32_t n_opts, int nacc,
                                     const double* __restrict__ partials, BatchOutputs out) {
-  const uint32_t o = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (o >= n_opts) return;
   const BatchOption& O = opts[o];
   double s[kAdjAcc];
+#pragma unroll
   for (int a = 0; a < kAdjAcc; ++a) s[a] = 0.0;
-  for (uint32_t i = O.item_begin; i < O.item_begin + O.item_count; ++i)
-    for (int a = 0; a < nacc; ++a) s[a] += partials[(size_t)i * nacc + a];
+  const uint32_t end = O.item_begin + O.item_count;
+  for (uint32_t i = O.item_begin + lane; i < end; i += 32)
+#pragma unroll
+    for (int a = 0; a < kAdjAcc; ++a)
+      if (a < nacc) s[a] += partials[(size_t)i * nacc + a];
+#pragma unroll
+  for (int k = 16; k >= 1; k >>= 1)
+#pragma unroll
+    for (int a = 0; a < kAdjAcc; ++a)
+      if (a < nacc) s[a] += __shfl_xor_sync(kFull, s[a], k);
+  if (lane != 0) return;
   const double n = (double)O.paths, inv_n = 1.0 / n;
   const double mean = s[0] * inv_n;
   const double price = O.disc * mean;
@@ -183,7 +215,9 @@ BatchKernel batch_kernel(const BatchLaunch& B) {
 }
 
 size_t batch_smem(const BatchLaunch& B) {
-  return B.adjoint && !B.gseg ? (size_t)(B.ckpt_rows + 3 * B.seg_rows) * B.tpb * sizeof(float) : 0;
+  if (B.adjoint && !B.gseg) return (size_t)(B.ckpt_rows + 3 * B.seg_rows) * B.tpb * sizeof(float);
+  const bool table = B.adjoint || (B.ppt == 2 && B.unroll == 1);
+  return table ? (size_t)B.tab_rows * (B.tpb / kWarp) * sizeof(uint4) : 0;
 }
 
 }  // namespace
@@ -195,7 +229,6 @@ void batch_variant(int v, bool adjoint, BatchLaunch* B) {
 }
 
 cudaError_t prepare_batch(const BatchLaunch& B) {
-  if (!B.adjoint || B.gseg) return cudaSuccess;
   return cudaFuncSetAttribute(batch_kernel(B), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem(B));
 }
 
@@ -230,7 +263,7 @@ cudaError_t launch_batch(const BatchLaunch& B, const BatchOption* opts, const Ba
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int nacc = B.adjoint ? kAdjAcc : 2;
-  batch_reduce_kernel<<<(B.n_opts + 127) / 128, 128, 0, stream>>>(opts, B.n_opts, nacc, partials, out);
+  batch_reduce_kernel<<<(B.n_opts + 3) / 4, 128, 0, stream>>>(opts, B.n_opts, nacc, partials, out);
   return cudaGetLastError();
 }
 
