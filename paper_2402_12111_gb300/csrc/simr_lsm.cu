@@ -39,6 +39,7 @@
 // resolve.  The coefficients are reported in x and y (converted in FP64).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdlib>
 
@@ -55,6 +56,10 @@ constexpr int kNMono = 15;  // x^a y^b, a + b <= 4
 constexpr int kNB = 6;      // basis functions
 constexpr int kNReg = kNMono + kNB;
 constexpr int kLsmPpt = 2;
+#ifndef SIMR_LSM_WARPS
+#define SIMR_LSM_WARPS 24  // of the path kernel, per SM
+#endif
+constexpr int kLsmPathTpb = kWarp * SIMR_LSM_WARPS;
 
 // Double-float sums: hi + lo carries about 48 significant bits, with FP32
 // arithmetic only (GB300's FP64 rate makes each FP64 warp instruction cost tens
@@ -77,88 +82,63 @@ __device__ __forceinline__ float lsm_payoff(bool put, float S, float K) {
   return put ? fmaxf(K - S, 0.0f) : fmaxf(S - K, 0.0f);
 }
 
-// One step of the thread's two paths from their (variance, log-spot) words,
-// paired in packed FP32 (simulate_two's arithmetic, or step_qem2 for QE-M).
+// Path kernel: states at the exercise dates, maturity cash flow.  One block per SM;
+// its warps take the block's 64-path batches from a counter in shared memory and
+// step two paths per thread through the pipelined loop.  Dynamic shared memory: the
+// step pairs' counter table (n_tab entries, 0: none).  252 dates x 2^20 paths.
 template <bool QEM>
-__device__ __forceinline__ void step_two(const LsmLaunch& L, uint32_t wv0, uint32_t wx0, uint32_t wv1, uint32_t wx1,
-                                         float (&v)[kLsmPpt], float (&x)[kLsmPpt], float (&comp)[kLsmPpt]) {
-  static_assert(kLsmPpt == 2, "two paths per thread");
-  const float2 xv = centered_uniform2(wv0, wv1);
-  const float2 zv = norminv_centered2(xv);
-  const float2 zx = norminv_centered2(centered_uniform2(wx0, wx1));
-  float2 vv = make_float2(v[0], v[1]), xx = make_float2(x[0], x[1]), cc = make_float2(comp[0], comp[1]);
-  if constexpr (QEM)
-    step_qem2(L.sc, L.qm, xv, zv, zx, vv, xx, cc);
-  else
-    step_base2<false>(L.sc, xv, zv, zx, vv, xx, cc);
-  v[0] = vv.x;
-  v[1] = vv.y;
-  x[0] = xx.x;
-  x[1] = xx.y;
-  comp[0] = cc.x;
-  comp[1] = cc.y;
-}
-
-// Path kernel: states at the exercise dates, maturity cash flow.
-template <bool QEM>
-__global__ void __launch_bounds__(kLsmTpb) lsm_paths_kernel(const __grid_constant__ LsmLaunch L,
-                                                            float* __restrict__ S_out, float* __restrict__ V_out,
-                                                            float* __restrict__ cash, int32_t* __restrict__ stop) {
+__global__ void __launch_bounds__(kLsmPathTpb, 1) lsm_paths_kernel(const __grid_constant__ LsmLaunch L, int n_tab,
+                                                                   float* __restrict__ S_out, float* __restrict__ V_out,
+                                                                   float* __restrict__ cash, int32_t* __restrict__ stop) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned s_next;
+  uint4* tab = reinterpret_cast<uint4*>(smem_raw);
   const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) s_next = 0u;
+  for (int p = threadIdx.x; p < n_tab; p += blockDim.x) tab[p] = philox_pair_entry(p, L.option_index, 0u, L.rk);
+  __syncthreads();
   const uint64_t per = (uint64_t)kWarp * kLsmPpt;
   const uint64_t batches = (L.paths + per - 1) / per;
-  const uint64_t n_warps = (uint64_t)gridDim.x * kLsmWarps;
+  const uint64_t block0 = batches / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, batches % gridDim.x);
+  const unsigned nb = (unsigned)(batches / gridDim.x + (blockIdx.x < batches % gridDim.x ? 1 : 0));
   const bool put = L.is_put != 0;
-  for (uint64_t bt = (uint64_t)blockIdx.x * kLsmWarps + (threadIdx.x >> 5); bt < batches; bt += n_warps) {
-    uint64_t idx[kLsmPpt];
-    PhiloxLane pl[kLsmPpt];
-    float v[kLsmPpt], x[kLsmPpt], comp[kLsmPpt];
-#pragma unroll
-    for (int j = 0; j < kLsmPpt; ++j) {
-      idx[j] = bt * per + (uint64_t)j * kWarp + lane;
-      pl[j] = philox_lane(idx[j], L.rk);
-      v[j] = L.sc.v0;
-      x[j] = 0.0f;
-      comp[j] = 0.0f;
-    }
-    int cnt = 0;
+  while (true) {
+    unsigned it = 0;
+    if (lane == 0) it = atomicAdd(&s_next, 1u);
+    it = __shfl_sync(kFull, it, 0);
+    if (it >= nb) break;
+    const uint64_t i0 = (block0 + it) * per + lane, i1 = i0 + kWarp;
+    const bool a0 = i0 < L.paths, a1 = i1 < L.paths;
+    float2 v, x, comp;
+    uint32_t cnt = 0;
     size_t row = 0;  // offset of the next date's row
-    auto record = [&]() {
-#pragma unroll
-      for (int j = 0; j < kLsmPpt; ++j) {
-        if (idx[j] < L.paths) {
-          S_out[row + idx[j]] = terminal_spot(L.S0, x[j], comp[j]);
-          V_out[row + idx[j]] = v[j];
-        }
+    auto record = [&](uint32_t) {
+      if (++cnt != (uint32_t)L.every) return;
+      cnt = 0;
+      if (a0) {
+        S_out[row + i0] = terminal_spot(L.S0, x.x, comp.x);
+        V_out[row + i0] = v.x;
+      }
+      if (a1) {
+        S_out[row + i1] = terminal_spot(L.S0, x.y, comp.y);
+        V_out[row + i1] = v.y;
       }
       row += L.pitch;
     };
-    for (uint32_t p = 0; 2 * p < L.steps; ++p) {
-      uint4 w[kLsmPpt];
-      const PhiloxCtr u = philox_ctr(p, L.option_index, L.rk);
-#pragma unroll
-      for (int j = 0; j < kLsmPpt; ++j) w[j] = philox_draw(pl[j], u, L.rk);
-      step_two<QEM>(L, w[0].x, w[0].y, w[1].x, w[1].y, v, x, comp);
-      if (++cnt == L.every) {
-        cnt = 0;
-        record();
-      }
-      if (2 * p + 1 < L.steps) {
-        step_two<QEM>(L, w[0].z, w[0].w, w[1].z, w[1].w, v, x, comp);
-        if (++cnt == L.every) {
-          cnt = 0;
-          record();
-        }
-      }
-    }
+    if (n_tab)
+      simulate_two_pipe<QEM, true>(L.sc, L.steps, L.option_index, L.rk, tab, i0, i1, v, x, comp, L.qm, record);
+    else
+      simulate_two_pipe<QEM, false>(L.sc, L.steps, L.option_index, L.rk, tab, i0, i1, v, x, comp, L.qm, record);
     // the last date is the maturity: its payoff starts each path's cash flow
-#pragma unroll
-    for (int j = 0; j < kLsmPpt; ++j) {
-      if (idx[j] < L.paths) {
-        const float h = lsm_payoff(put, terminal_spot(L.S0, x[j], comp[j]), L.K);
-        cash[idx[j]] = h;
-        stop[idx[j]] = h > 0.0f ? L.n_ex - 1 : -1;
-      }
+    if (a0) {
+      const float h = lsm_payoff(put, terminal_spot(L.S0, x.x, comp.x), L.K);
+      cash[i0] = h;
+      stop[i0] = h > 0.0f ? L.n_ex - 1 : -1;
+    }
+    if (a1) {
+      const float h = lsm_payoff(put, terminal_spot(L.S0, x.y, comp.y), L.K);
+      cash[i1] = h;
+      stop[i1] = h > 0.0f ? L.n_ex - 1 : -1;
     }
   }
 }
@@ -979,17 +959,17 @@ cudaError_t try_sweep(const LsmLaunch& L, const LsmBuffers& B, const LsmSweep& Y
 }  // namespace
 
 cudaError_t launch_lsm(const LsmLaunch& L, const LsmBuffers& B, int num_sms, cudaStream_t stream) {
-  int per_sm = 0;
+  // one block per SM; fewer warps where they get under four batches each, as many as make the rounds even
+  const uint64_t per = (uint64_t)kWarp * kLsmPpt, batches = (L.paths + per - 1) / per;
+  const uint64_t grid = std::min<uint64_t>(num_sms, batches), most = (batches + grid - 1) / grid;
+  uint64_t warps = std::min<uint64_t>(SIMR_LSM_WARPS, most);
+  const uint64_t rounds = (most + warps - 1) / warps;
+  if (rounds == 2) warps = (most + rounds - 1) / rounds;
+  const uint64_t pairs = (uint64_t)L.steps / 2 + 2;
+  const int n_tab = pairs <= 2048 ? (int)pairs : 0;  // (at most 2^31 paths: the high counter word is 0)
   auto pk = L.scheme == 1 ? lsm_paths_kernel<true> : lsm_paths_kernel<false>;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pk, kLsmTpb, 0);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const uint64_t batches = (L.paths + (uint64_t)kWarp * kLsmPpt - 1) / ((uint64_t)kWarp * kLsmPpt);
-  uint64_t grid = (uint64_t)num_sms * per_sm;
-  const uint64_t need = (batches + kLsmWarps - 1) / kLsmWarps;
-  if (grid > need) grid = need;
-  pk<<<(unsigned)grid, kLsmTpb, 0, stream>>>(L, B.S, B.V, B.cash, B.stop);
-  e = cudaGetLastError();
+  pk<<<(unsigned)grid, (unsigned)(kWarp * warps), n_tab * sizeof(uint4), stream>>>(L, n_tab, B.S, B.V, B.cash, B.stop);
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
 
   bool swept = false;
