@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(128, SIMR_ADJ_MINB_SMEM) heston_adjoint_kernel
       pth[j] = L.path_begin + local;
     }
     float x[PPT], comp[PPT], g[PPT][5], S[PPT];
-    path_adjoint_ppt<PPT, SegShared, true, QEM>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
-                                                SegShared{sbuf, A.ckpt_every}, x, comp, g, L.qm);
+    path_adjoint_ppt<PPT, SegShared, QEM>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
+                                                SegShared{sbuf}, x, comp, g, L.qm);
 #pragma unroll
     for (int j = 0; j < PPT; ++j) S[j] = terminal_spot(L.S0, x[j], comp[j]);
 
@@ -239,7 +239,8 @@ __global__ void __launch_bounds__(128, SIMR_ADJ_MINB_SMEM) heston_adjoint_kernel
 // path-step, 33 of them packed).  252 steps x 2^20 paths x 32 strikes: 2,072 us with
 // five blocks of 128 that strode over the batches (and one thread per sum over 760
 // block rows at the end), 1,740 with items at 20 warps, 1,598 at 24 (80 registers;
-// 28 and 32 warps spill: 2,040 and 2,080); QE-M 948 -> 680 us at 2^18 paths.
+// 28 and 32 warps spill: 2,040 and 2,080), 1,388 with the segments in warp slabs
+// (SegWarp) and no selects on the common path; QE-M 948 -> 556 us at 2^18 paths.
 template <int TILE, bool QEM>
 __global__ void __launch_bounds__(kWarp * (QEM ? SIMR_ADJ_QEM_WARPS : SIMR_ADJ_WARPS), 1)
     heston_adjoint_seg_kernel(const __grid_constant__ PathLaunch L, const __grid_constant__ AdjConst A,
@@ -285,12 +286,12 @@ __global__ void __launch_bounds__(kWarp * (QEM ? SIMR_ADJ_QEM_WARPS : SIMR_ADJ_W
       const bool act[1] = {local < L.path_count};
       const uint64_t pth[1] = {L.path_begin + local};
       float x[1], comp[1], g[1][5];
-      const SegGlobal seg{gseg, (long long)blockIdx.x * bd + tid, A.ckpt_every, (long long)ck_stride};
+      const SegWarp seg{gseg, A.ckpt_every};
       if (tab)
-        path_adjoint_ppt<1, SegGlobal, true, QEM, true>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
+        path_adjoint_ppt<1, SegWarp, QEM, true>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
                                                         seg, x, comp, g, L.qm, tab);
       else
-        path_adjoint_ppt<1, SegGlobal, true, QEM, false>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
+        path_adjoint_ppt<1, SegWarp, QEM, false>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ck, ck_stride,
                                                          seg, x, comp, g, L.qm);
       const float S[1] = {terminal_spot(L.S0, x[0], comp[0])};
       if (TILE == 1) {
@@ -329,8 +330,8 @@ __global__ void __launch_bounds__(128) heston_paths_adjoint_kernel(const __grid_
   if (i >= L.path_count) return;  // no block-wide synchronisation below
   float x[1], comp[1], g[1][5];
   const uint64_t pth[1] = {L.path_begin + i};
-  path_adjoint_ppt<1, SegShared, true, QEM>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ckpt + tid, bd,
-                                            SegShared{ckpt + (A.n_seg - 1) * bd, A.ckpt_every}, x, comp, g, L.qm);
+  path_adjoint_ppt<1, SegShared, QEM>(L.sc[0], A, L.steps, L.option_index, L.rk, pth, ckpt + tid, bd,
+                                            SegShared{ckpt + (A.n_seg - 1) * bd}, x, comp, g, L.qm);
   x_T[i] = x[0] - comp[0];
 #pragma unroll
   for (int j = 0; j < 5; ++j) grad[i * 5 + j] = g[0][j];

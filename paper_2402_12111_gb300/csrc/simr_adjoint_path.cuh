@@ -9,7 +9,7 @@
 #include "simr_internal.h"
 
 #ifndef SIMR_ADJ_PREFETCH
-#define SIMR_ADJ_PREFETCH 4  // steps ahead the reverse sweep asks global segment data into L2 (4-32 within 2%)
+#define SIMR_ADJ_PREFETCH 2  // pairs of steps ahead the reverse sweep asks global segment data into L2
 #endif
 
 namespace simr {
@@ -204,17 +204,16 @@ __device__ __forceinline__ void adjoint_step(const ScenConst& c, float theta, fl
 }
 
 // adjoint_step2 for a warp whose every lane takes the quadratic branch in both
-// steps (the same operations as its general form, without the exponential
-// branch's code and registers).
+// steps and has v + v' > 0 (the same operations as its general form, without the
+// exponential branch's code and registers and the selects at v + v' = 0).
 __device__ __forceinline__ void adjoint_step2_quad(const ScenConst& c, float theta, float c1, float2 vc, float2 vn,
-                                                   float2 d, float2 zx, float2 m, float2 m2, float2 rs2h, float2 t,
+                                                   float2 d, float2 zx, float2 m, float2 s, float2 rs2h, float2 t,
                                                    AdjSums& a) {
-  const float2 s = p_add(vc, vn);
   const float2 rq = make_float2(rsqrt_approx(s.x), rsqrt_approx(s.y));
-  const float2 sq = p_mul(s, rq);
+  const float2 q = p_mul(s, rq);
   const float2 hq = p_mul(p_mul(p_bc(0.5f * c.sK3), zx), rq);
-  const float2 q = make_float2(s.x > 0.0f ? sq.x : 0.0f, s.y > 0.0f ? sq.y : 0.0f);
-  const float2 hzc = p_add(make_float2(s.x > 0.0f ? hq.x : 0.0f, s.y > 0.0f ? hq.y : 0.0f), p_bc(c.Cv));
+  // (scalar: a packed product and sum side by side come out fused)
+  const float2 hzc = make_float2(__fadd_rn(hq.x, c.Cv), __fadd_rn(hq.y, c.Cv));
   const float2 hzcd = p_sub(hzc, p_bc(c.Cd));
   const float2 tmv = p_sub(p_bc(theta), vc);
   const float2 tt = p_fma(t, t, p_mul(t, p_bc(-1.0f)));
@@ -265,12 +264,12 @@ __device__ __forceinline__ void adjoint_step2(const ScenConst& c, float theta, f
   const float2 rs2h = p_rcp(s2h);
   const float2 t = p_mul(m2, rs2h);  // qe_t, lane for lane
   const bool qx = t.x > kQuadT, qy = t.y > kQuadT;
-  if (__all_sync(0xffffffffu, qx && qy)) {  // the whole warp in the quadratic branch
-    adjoint_step2_quad(c, theta, c1, vc, vn, d, zx, m, m2, rs2h, t, a);
+  const float2 s = p_add(vc, vn);
+  if (__all_sync(0xffffffffu, qx && qy && s.x > 0.0f && s.y > 0.0f)) {  // the whole warp on the common path
+    adjoint_step2_quad(c, theta, c1, vc, vn, d, zx, m, s, rs2h, t, a);
     return;
   }
   // adj_common_pre, paired
-  const float2 s = p_add(vc, vn);
   const float2 rq = make_float2(rsqrt_approx(s.x), rsqrt_approx(s.y));
   const float2 sq = p_mul(s, rq);
   const float2 hq = p_mul(p_mul(p_bc(0.5f * c.sK3), zx), rq);
@@ -461,24 +460,6 @@ __device__ __forceinline__ void adjoint_step_qem(const ScenConst& c, const QemCo
   }
 }
 
-// The draw the reverse step of state v needs: Z_V in the quadratic branch,
-// 1 - U_V otherwise (same branch test as the forward step).
-__device__ __forceinline__ float branch_draw(const ScenConst& c, float v, float xv, float zv) {
-  const float m = fmaf(v, c.E, c.thE);
-  const float s2h = fmaf(v, c.h1, c.h2);
-  return qe_t(m * m, s2h) > kQuadT ? zv : one_minus_u(xv);
-}
-
-// One step of the recompute pass: the stored data -- (state, branch draw) as one
-// pair and Z_X -- and the next state, from the step's centred variance uniform and
-// its two normals.
-__device__ __forceinline__ void keep_step(const ScenConst& c, float xv, float zv, float zx, float2* bvd, float* bz,
-                                          float& v) {
-  *bvd = make_float2(v, branch_draw(c, v, xv, zv));
-  *bz = zx;
-  v = qe_only(c, v, xv, zv);
-}
-
 // The draws of a step pair: 2 U_V - 1, Z_V and Z_X, lane x the even step's.
 struct PairDraw {
   float2 xv, zv, zx;
@@ -495,53 +476,75 @@ __device__ __forceinline__ void pair_draw_fix(PairDraw& d, float2 xx, float2 wcv
   norminv_fix2(xx, wcx, d.zx);
 }
 
-// keep_step of the even step of a pair and the draws of the next pair, from its
-// words: independent of each other, and what leaves the common path (a tail
-// normal, the exponential branch) is redone behind one test.
+// The next state of one step, and its stored (state, branch draw) pair in vd: the
+// quadratic branch straight through, the exponential branch (quad false) by keep_fix.
+struct KeepStep {
+  float m, s2h, m2;
+  bool quad;
+};
+__device__ __forceinline__ KeepStep keep_try(const ScenConst& c, float v, float zv, float2& vd, float& vn) {
+  KeepStep k;
+  k.m = fmaf(v, c.E, c.thE);
+  k.s2h = fmaf(v, c.h1, c.h2);
+  k.m2 = __fmul_rn(k.m, k.m);
+  const float t = qe_t(k.m2, k.s2h);
+  float dl;
+  qe_quad_branch(k.m, t, zv, vn, dl);
+  vd = make_float2(v, zv);
+  k.quad = t > kQuadT;
+  return k;
+}
+__device__ __forceinline__ void keep_fix(const KeepStep& k, float xv, float2& vd, float& vn) {
+  float dl;
+  vd.y = one_minus_u(xv);
+  qe_exp_branch(k.m, k.s2h, k.m2, xv, vn, dl);
+}
+
+// The even step of a pair and the draws of the next pair, from its words:
+// independent of each other, and what leaves the common path (a tail normal, the
+// exponential branch) is redone behind one test.
 __device__ __forceinline__ void keep_step_pipe(const ScenConst& c, const PairDraw& d, const uint4& wn, PairDraw& dn,
-                                               float2* bvd, float* bz, float& v) {
-  const float m = fmaf(v, c.E, c.thE);
-  const float s2h = fmaf(v, c.h1, c.h2);
-  const float m2 = __fmul_rn(m, m);
-  const float t = qe_t(m2, s2h);
-  float vn, dl, dr = d.zv.x;
-  qe_quad_branch(m, t, d.zv.x, vn, dl);
-  const bool quad = t > kQuadT;
+                                               float2& vd, float& v) {
+  float vn;
+  const KeepStep k = keep_try(c, v, d.zv.x, vd, vn);
   float2 xx, wcv, wcx;
   const bool central = pair_draw_try(wn, dn, xx, wcv, wcx);
-  if (!(quad && central)) {
+  if (!(k.quad && central)) {
     pair_draw_fix(dn, xx, wcv, wcx);
-    if (!quad) {
-      dr = one_minus_u(d.xv.x);
-      qe_exp_branch(m, s2h, m2, d.xv.x, vn, dl);
-    }
+    if (!k.quad) keep_fix(k, d.xv.x, vd, vn);
   }
-  *bvd = make_float2(v, dr);
-  *bz = d.zx.x;
+  v = vn;
+}
+// The odd step of a pair.
+__device__ __forceinline__ void keep_step_odd(const ScenConst& c, const PairDraw& d, float2& vd, float& v) {
+  float vn;
+  const KeepStep k = keep_try(c, v, d.zv.y, vd, vn);
+  if (!k.quad) keep_fix(k, d.xv.y, vd, vn);
   v = vn;
 }
 
-// A thread's column of a segment buffer of `stride` columns (8-byte aligned):
-// `rows` (state, draw) float2 pairs at pairs[i * stride], then `rows` Z_X floats
-// at zx[i * stride].  SegShared: the block's buffer in shared memory, column
-// threadIdx.x of blockDim.x; SegGlobal: a grid-wide buffer in global memory,
-// column `col` (the thread's index in the grid) of `stride`.
+// A segment's stored steps, in pairs (2p, 2p + 1): each step's (state, branch draw)
+// as one float2 and the pair's two Z_X as another, three float2 rows kRow apart per
+// pair and pairs kPair rows apart.  SegShared: the block's buffer in shared memory,
+// one column per thread.  SegWarp: the warp's own slab in global memory, [pair][3][32
+// lanes] -- a warp's accesses are contiguous and every offset is a constant, where a
+// grid-wide [step][thread] array cost eight 64-bit address sums per step.
 struct SegShared {
   static constexpr bool kGlobal = false;
   float* base;
-  int rows;
-  __device__ __forceinline__ int stride() const { return (int)blockDim.x; }
   __device__ __forceinline__ float2* pairs() const { return reinterpret_cast<float2*>(base) + threadIdx.x; }
-  __device__ __forceinline__ float* zx() const { return base + 2 * rows * (int)blockDim.x + threadIdx.x; }
+  __device__ __forceinline__ int row() const { return (int)blockDim.x; }
 };
 
-struct SegGlobal {
+struct SegWarp {
   static constexpr bool kGlobal = true;
-  float* base;
-  long long col, rows, cols;
-  __device__ __forceinline__ long long stride() const { return cols; }
-  __device__ __forceinline__ float2* pairs() const { return reinterpret_cast<float2*>(base) + col; }
-  __device__ __forceinline__ float* zx() const { return base + 2 * rows * cols + col; }
+  float* base;  // the grid's buffer, 3 rows floats per thread
+  int rows;     // steps per segment (even)
+  __device__ __forceinline__ float2* pairs() const {
+    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    return reinterpret_cast<float2*>(base + warp * 96 * rows) + (threadIdx.x & 31);
+  }
+  static __device__ __forceinline__ constexpr int row() { return 32; }
 };
 
 // The FP64 map of the sweep's sums onto d x_T / d(v0, kappa, theta, sigma, rho).
@@ -574,30 +577,26 @@ __device__ __forceinline__ void adjoint_map(const AdjConst& A, const AdjSums& a,
 // thread's segment column S (at least k rows) -- then the steps are
 // differentiated backwards.  x_T (with its Kahan remainder) is summed on the
 // way; g = d x_T / d(v0, kappa, theta, sigma, rho).
-template <typename Seg, bool PAIRED, bool QEM, bool TAB>
+template <typename Seg, bool QEM, bool TAB>
 __device__ __forceinline__ void path_sweep(const ScenConst& c, const AdjConst& A, uint32_t N, uint32_t option,
                                            const uint32_t (&rk)[10][2], const uint4* tab, const PhiloxLane& pl0,
                                            const float* ck, int cstride, float v_last, const Seg& S,
                                            float& x_out, float& comp_out, float (&g)[5], const QemConst& qm) {
-  using I = decltype(S.stride());
   const float theta = A.theta;
   const float c1 = c.h1 + c.h1;  // s^2 = v c1 + c2
   const uint32_t k = (uint32_t)A.ckpt_every;
   const int n_seg = A.n_seg;
   const PhiloxLane pl[1] = {pl0};
   AdjSums as = AdjSums{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  float2* s01 = S.pairs();
-  float* s2 = S.zx();
-  const I bd = S.stride();
+  float2* const first = S.pairs();
+  const int r1 = S.row(), r2 = 2 * r1, r3 = 3 * r1;
   float ck_next = v_last;
   for (int sgi = n_seg - 1; sgi >= 0; --sgi) {
     const uint32_t n0 = (uint32_t)sgi * k, n1 = min(n0 + k, N);
     float vv = ck_next;
     if (sgi > 0) ck_next = ck[(sgi - 1) * cstride];
-    // recompute v_n0 .. v_n1 and keep the draws: rows 2 (p - n0/2) and the next of
-    // this thread's column, by pointers stepped two rows per pair (n0 is even)
-    float2* wp = s01;
-    float* wz = s2;
+    // recompute v_n0 .. v_n1 and keep the draws (n0 is even)
+    float2* wp = first;
     PairDraw d, dn;
     uint4 w[1];
     philox_draws<TAB, 1>(tab, n0 / 2, option, rk, pl, w);
@@ -606,105 +605,61 @@ __device__ __forceinline__ void path_sweep(const ScenConst& c, const AdjConst& A
       if (!pair_draw_try(w[0], d, xx, wcv, wcx)) pair_draw_fix(d, xx, wcv, wcx);
     }
 #pragma unroll 1
-    for (uint32_t p = n0 / 2; 2 * p < n1; ++p, wp += 2 * bd, wz += 2 * bd) {
+    for (uint32_t p = n0 / 2; 2 * p < n1; ++p, wp += r3) {
       philox_draws<TAB, 1>(tab, p + 1, option, rk, pl, w);  // (the pair past the segment is drawn and not used)
-      keep_step_pipe(c, d, w[0], dn, wp, wz, vv);
-      if (2 * p + 1 < n1) keep_step(c, d.xv.y, d.zv.y, d.zx.y, wp + bd, wz + bd, vv);
+      float2 vd;
+      keep_step_pipe(c, d, w[0], dn, vd, vv);
+      wp[0] = vd;
+      wp[r2] = d.zx;
+      if (2 * p + 1 < n1) {
+        keep_step_odd(c, d, vd, vv);
+        wp[r1] = vd;
+      }
       d = dn;
     }
     float vnext = vv;  // v_{n1}
-    // the reverse steps read row i by pointers rp, rz stepped down from the top row
-    int i = (int)(n1 - n0) - 1;
-    const float2* rp = s01 + (I)i * bd;
-    const float* rz = s2 + (I)i * bd;
-    if constexpr (QEM) {
-      for (; i >= 0; --i, rp -= bd, rz -= bd) {
-        const float2 vd = rp[0];
-        adjoint_step_qem(c, qm, theta, c1, vd.x, vnext, vd.y, rz[0], as);
-        vnext = vd.x;
+    // the reverse steps, from the top pair down
+    int left = (int)(n1 - n0 + 1) / 2;
+    const float2* rp = first + (left - 1) * (decltype(r3))r3;
+    float2 a = rp[0], b = rp[r1], z = rp[r2];
+    if ((n1 - n0) & 1u) {  // an odd count: the last step alone
+      if constexpr (QEM)
+        adjoint_step_qem(c, qm, theta, c1, a.x, vnext, a.y, z.x, as);
+      else
+        adjoint_step(c, theta, c1, a.x, vnext, a.y, z.x, as);
+      vnext = a.x;
+      --left;
+      rp -= r3;
+      if (left > 0) {
+        a = rp[0];
+        b = rp[r1];
+        z = rp[r2];
       }
-    } else if constexpr (PAIRED) {
-      if constexpr (Seg::kGlobal) {
-        // global memory: the steps in pairs (n, n - 1) from the top, each pair's
-        // data loaded one pair ahead into registers and asked into L2
-        // kPrefetchSteps steps ahead
-        constexpr int kPrefetchSteps = SIMR_ADJ_PREFETCH;
-        const I o2 = 2 * bd, o3 = 3 * bd, f2 = (2 + kPrefetchSteps) * bd, f3 = (3 + kPrefetchSteps) * bd;
-        float2 pa = rp[0], pb = make_float2(0.0f, 0.0f);
-        float za = rz[0], zb = 0.0f;
-        if (i >= 1) {
-          pb = rp[-bd];
-          zb = rz[-bd];
+    }
+#pragma unroll 1
+    for (; left > 0; --left, rp -= r3) {
+      const float2 ca = a, cb = b, cz = z;
+      if (left > 1) {  // the next pair's data into registers
+        a = rp[-r3];
+        b = rp[r1 - r3];
+        z = rp[r2 - r3];
+      }
+      if constexpr (Seg::kGlobal) {  // and asked into L2 kPrefetch pairs further ahead
+        constexpr int kPrefetch = SIMR_ADJ_PREFETCH;
+        if (left > 1 + kPrefetch) {
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(rp - (1 + kPrefetch) * r3));
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + r1 - (1 + kPrefetch) * r3));
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + r2 - (1 + kPrefetch) * r3));
         }
-        for (; i >= 1; i -= 2, rp -= o2, rz -= o2) {
-          const float2 ca = pa, cb = pb;
-          const float cza = za, czb = zb;
-          if (i - 2 - kPrefetchSteps >= 0) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(rp - f2));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(rz - f2));
-          }
-          if (i - 3 - kPrefetchSteps >= 0) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(rp - f3));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(rz - f3));
-          }
-          if (i >= 2) {
-            pa = rp[-o2];
-            za = rz[-o2];
-          }
-          if (i >= 3) {
-            pb = rp[-o3];
-            zb = rz[-o3];
-          }
-          adjoint_step2(c, theta, c1, make_float2(ca.x, cb.x), make_float2(vnext, ca.x), make_float2(ca.y, cb.y),
-                        make_float2(cza, czb), as);
-          vnext = cb.x;
-        }
-        if (i == 0) {  // an odd count: the last step alone (loaded as pa)
-          adjoint_step(c, theta, c1, pa.x, vnext, pa.y, za, as);
-          vnext = pa.x;
-        }
+      }
+      if constexpr (QEM) {
+        adjoint_step_qem(c, qm, theta, c1, cb.x, vnext, cb.y, cz.y, as);
+        adjoint_step_qem(c, qm, theta, c1, ca.x, cb.x, ca.y, cz.x, as);
       } else {
-        for (; i >= 1; i -= 2, rp -= 2 * bd, rz -= 2 * bd) {
-          const float2 ca = rp[0], cb = rp[-bd];
-          adjoint_step2(c, theta, c1, make_float2(ca.x, cb.x), make_float2(vnext, ca.x), make_float2(ca.y, cb.y),
-                        make_float2(rz[0], rz[-bd]), as);
-          vnext = cb.x;
-        }
-        if (i == 0) {
-          const float2 vd = s01[0];
-          adjoint_step(c, theta, c1, vd.x, vnext, vd.y, s2[0], as);
-          vnext = vd.x;
-        }
+        adjoint_step2(c, theta, c1, make_float2(cb.x, ca.x), make_float2(vnext, cb.x), make_float2(cb.y, ca.y),
+                      make_float2(cz.y, cz.x), as);
       }
-    } else {
-      if constexpr (Seg::kGlobal) {
-        // global memory: each step's data loaded one step ahead into registers,
-        // and asked into L2 kPrefetchSteps steps ahead
-        constexpr int kPrefetchSteps = SIMR_ADJ_PREFETCH;
-        const I f = (I)kPrefetchSteps * bd;
-        float2 vd_n = rp[0];
-        float zx_n = rz[0];
-        for (; i >= 0; --i, rp -= bd, rz -= bd) {
-          const float2 vd = vd_n;
-          const float zx = zx_n;
-          if (i >= kPrefetchSteps) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(rp - f));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(rz - f));
-          }
-          if (i > 0) {
-            vd_n = rp[-bd];
-            zx_n = rz[-bd];
-          }
-          adjoint_step(c, theta, c1, vd.x, vnext, vd.y, zx, as);
-          vnext = vd.x;
-        }
-      } else {
-        for (; i >= 0; --i, rp -= bd, rz -= bd) {
-          const float2 vd = rp[0];
-          adjoint_step(c, theta, c1, vd.x, vnext, vd.y, rz[0], as);
-          vnext = vd.x;
-        }
-      }
+      vnext = ca.x;
     }
   }
   x_out = as.x;
@@ -721,7 +676,7 @@ __device__ __forceinline__ void path_sweep(const ScenConst& c, const AdjConst& A
 // Checkpoint (slot, path j) of this thread at ck[(slot * PPT + j) * ck_stride]
 // (n_seg - 1 slots; shared or global memory); S is this thread's segment column
 // (shared or global memory, at least k rows).
-template <int PPT, typename Seg, bool PAIRED = true, bool QEM = false, bool TAB = false>
+template <int PPT, typename Seg, bool QEM = false, bool TAB = false>
 __device__ __forceinline__ void path_adjoint_ppt(const ScenConst& c, const AdjConst& A, uint32_t N, uint32_t option,
                                                  const uint32_t (&rk)[10][2], const uint64_t (&path)[PPT], float* ck,
                                                  int ck_stride, const Seg& S, float (&x_out)[PPT],
@@ -765,7 +720,7 @@ __device__ __forceinline__ void path_adjoint_ppt(const ScenConst& c, const AdjCo
   }
 #pragma unroll
   for (int j = 0; j < PPT; ++j)
-    path_sweep<Seg, PAIRED, QEM, TAB>(c, A, N, option, rk, tab, pl[j], ck + j * ck_stride, PPT * ck_stride, v[j], S,
+    path_sweep<Seg, QEM, TAB>(c, A, N, option, rk, tab, pl[j], ck + j * ck_stride, PPT * ck_stride, v[j], S,
                                  x_out[j], comp_out[j], g[j], qm);
 }
 

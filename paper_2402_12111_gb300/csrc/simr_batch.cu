@@ -32,9 +32,6 @@ namespace {
 // registers; QE-M 8.7 ms against 8.9 at 640 threads on 16 options, QE the same),
 // price books with the pipelined pair of paths 512 (7.5 -> 6.6 ms for 64 options,
 // QE-M 5.35 -> 3.4 ms for 16; 640 and 768 within 3%).
-#ifndef SIMR_BOOK_PAIRED
-#define SIMR_BOOK_PAIRED true  // reverse steps in pairs (one at a time: 351 ms against 311 for the book)
-#endif
 #ifndef SIMR_BOOK_ADJ_THREADS
 #define SIMR_BOOK_ADJ_THREADS 768
 #endif
@@ -90,14 +87,11 @@ __global__ void __launch_bounds__(TPB, ADJ ? SIMR_BOOK_ADJ_THREADS / TPB : PPT =
         // arrays of seg_rows rows (the largest over the book), so threads on
         // options with different checkpoint intervals never overlap
         if constexpr (GSEG)  // one segment: no checkpoints are read or written
-          path_adjoint_ppt<1, SegGlobal, SIMR_BOOK_PAIRED, QEM, true>(
-              c, O.A, steps, oidx, B.rk, pth, B.gseg, 0,
-              SegGlobal{B.gseg, (long long)blockIdx.x * bd + tid, B.seg_rows, (long long)gridDim.x * bd}, x, comp,
-              g, O.qm, tab);
+          path_adjoint_ppt<1, SegWarp, QEM, true>(c, O.A, steps, oidx, B.rk, pth, B.gseg, 0, SegWarp{B.gseg, B.seg_rows},
+                                                  x, comp, g, O.qm, tab);
         else
-          path_adjoint_ppt<1, SegShared, SIMR_BOOK_PAIRED, QEM>(c, O.A, steps, oidx, B.rk, pth, smem_f + tid, bd,
-                                                                SegShared{smem_f + B.ckpt_rows * bd, B.seg_rows},
-                                                                x, comp, g, O.qm);
+          path_adjoint_ppt<1, SegShared, QEM>(c, O.A, steps, oidx, B.rk, pth, smem_f + tid, bd,
+                                              SegShared{smem_f + B.ckpt_rows * bd}, x, comp, g, O.qm);
         const float S = terminal_spot(S0, x[0], comp[0]);
 #pragma unroll
         for (int a = 0; a < NACC; ++a) terms[a] = active ? adj_term(a, put, S, K, g[0], O.invS0, O.T) : 0.0f;
