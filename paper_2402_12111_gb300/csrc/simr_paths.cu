@@ -33,11 +33,12 @@
 #include "simr_internal.h"
 #include "simr_reduce.cuh"
 
-// Tuning knobs (compile-time): warps per SM of the pricing and the 3- and
-// 5-scenario kernels.  Measured at 252 steps x 2^20 paths: pricing 789 / 777 /
-// 789 us at 24 / 28 / 32 warps; 5 scenarios 2,446 / 2,270 / 2,270 us at 20 / 28 / 32.
-// QE-M pricing 285 / 289 / 242 us at 24 / 28 / 32 (101 steps x 300,007 paths x 40
-// strikes: 31 batches a block).
+// Tuning knobs (compile-time): warps per SM.  Measured at 252 steps x 2^20 paths:
+// pricing 770 / 785 / 786 us at 24 / 28 / 32 warps (pipelined loop); 5 scenarios
+// 2,214 / 2,171 / 2,157 / 2,169 us at 20 / 24 / 28 / 32; 11 scenarios (365 x 250,001)
+// 1,707 / 1,728 / 1,918 us at 16 / 20 / 24; 3 scenarios (one strike, 64 x 65,536)
+// 41.6 / 42.2 / 42.4 us at 20 / 24 / 32.  QE-M pricing 285 / 289 / 242 us at 24 /
+// 28 / 32 (101 x 300,007 x 40 strikes: 31 batches a block), before the pipelined loop.
 #ifndef SIMR_PRICE_WARPS
 #define SIMR_PRICE_WARPS 24
 #endif
@@ -45,7 +46,10 @@
 #define SIMR_QEM_WARPS 32
 #endif
 #ifndef SIMR_FD3_WARPS
-#define SIMR_FD3_WARPS 32
+#define SIMR_FD3_WARPS 24
+#endif
+#ifndef SIMR_FD11_WARPS
+#define SIMR_FD11_WARPS 16
 #endif
 #ifndef SIMR_FD5_WARPS
 #define SIMR_FD5_WARPS 28
@@ -104,6 +108,96 @@ __device__ __forceinline__ float resim_term(const PathLaunch& L, int up, int dn,
   return fmaf(ru, fu, fmaf(-rd, fd, fu - fd));
 }
 
+// The moments of the scenario pair (2P + 1, 2P + 2): the base's constants for the
+// v0 bumps (P < NV / 2), plus the pair's own deltas for the others.
+template <int NV>
+__device__ __forceinline__ void pair_moments(const PathLaunch& L, int P, float2 v, float2& m, float2& s2h) {
+  const ScenConst& b = L.sc[0];
+  if (2 * P + 2 <= NV) {
+    m = p_add(p_mul(v, p_bc(b.E)), p_bc(b.thE));
+    s2h = p_add(p_mul(v, p_bc(b.h1)), p_bc(b.h2));
+  } else {
+    const ScenConst2& d = L.pair2[P];
+    m = p_add(p_fma(v, p_bc(b.E), p_fma(v, d.E, d.thE)), p_bc(b.thE));
+    s2h = p_add(p_fma(v, p_bc(b.h1), p_fma(v, d.h1, d.h2)), p_bc(b.h2));
+  }
+}
+
+// One QE step of the base and its scenario pairs, lane for lane step_base<true> and
+// step_bumped: every chain's quadratic branch side by side, then one test for the
+// exponential branch, whose lanes are redone chain by chain.  (A test per chain kept
+// them apart: 252 steps x 2^20 paths x 32 strikes, 5 scenarios 2,230 -> 2,157 us; 11
+// scenarios at 365 x 250,001 x 21 1,806 -> 1,707.)
+template <int NS, int NV>
+__device__ __forceinline__ void step_merged(const PathLaunch& L, float xv, float zv, float zx, float (&v)[NS],
+                                            float (&x)[NS], float (&c)[NS]) {
+  constexpr int NP = (NS - 1) / 2;
+  const ScenConst& b = L.sc[0];
+  const float m0 = __fadd_rn(__fmul_rn(v[0], b.E), b.thE);
+  const float s0 = __fadd_rn(__fmul_rn(v[0], b.h1), b.h2);
+  const float m20 = __fmul_rn(m0, m0), t0 = qe_t(m20, s0);
+  float vn0, dl0;
+  qe_quad_branch(m0, t0, zv, vn0, dl0);
+  bool quad = t0 > kQuadT;
+  float2 vn[NP], dl[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    float2 m, s2h, m2, t;
+    pair_moments<NV>(L, p, make_float2(v[2 * p + 1], v[2 * p + 2]), m, s2h);
+    quad &= qe_try2(m, s2h, p_bc(zv), m2, t, vn[p], dl[p]);
+  }
+  if (!quad) {
+    if (!(t0 > kQuadT)) qe_exp_branch(m0, s0, m20, xv, vn0, dl0);
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      float2 m, s2h;
+      pair_moments<NV>(L, p, make_float2(v[2 * p + 1], v[2 * p + 2]), m, s2h);
+      const float2 m2 = p_mul(m, m);
+      qe_fix2(m, s2h, m2, p_mul(m2, p_rcp(s2h)), p_bc(xv), vn[p], dl[p]);
+    }
+  }
+  {
+    const float s = __fadd_rn(v[0], vn0);
+    float inc = __fmaf_rn(b.Cv, s, b.C0);
+    inc = __fmaf_rn(-b.Cd, v[0], inc);
+    inc = __fmaf_rn(b.Cdl, dl0, inc);
+    inc = __fmaf_rn(__fmul_rn(b.sK3, sqrt_approx(s)), zx, inc);
+    const float y = __fsub_rn(inc, c[0]);
+    const float t = __fadd_rn(x[0], y);
+    c[0] = __fsub_rn(__fsub_rn(t, x[0]), y);
+    x[0] = t;
+    v[0] = vn0;
+  }
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const float2 vv = make_float2(v[2 * p + 1], v[2 * p + 2]), xx = make_float2(x[2 * p + 1], x[2 * p + 2]),
+                 cc = make_float2(c[2 * p + 1], c[2 * p + 2]);
+    const float2 s = p_add(vv, vn[p]);
+    const float2 q = p_sqrt(s);
+    float2 inc = p_fma(p_bc(b.Cv), s, p_bc(b.C0));
+    inc = p_fma(p_bc(-b.Cd), vv, inc);
+    inc = p_fma(p_bc(b.Cdl), dl[p], inc);
+    inc = p_fma(p_mul(p_bc(b.sK3), q), p_bc(zx), inc);
+    if (2 * p + 2 > NV) {
+      const ScenConst2& d = L.pair2[p];
+      float2 sm = p_fma(d.Cv, s, d.C0);
+      sm = p_fma(d.mCd, vv, sm);
+      sm = p_fma(d.Cdl, dl[p], sm);
+      sm = p_fma(p_mul(d.sK3, q), p_bc(zx), sm);
+      inc = p_add(inc, sm);
+    }
+    const float2 y = p_sub(inc, cc);
+    const float2 t = p_add(xx, y);
+    const float2 cn = p_sub(p_sub(t, xx), y);
+    c[2 * p + 1] = cn.x;
+    c[2 * p + 2] = cn.y;
+    x[2 * p + 1] = t.x;
+    x[2 * p + 2] = t.y;
+    v[2 * p + 1] = vn[p].x;
+    v[2 * p + 2] = vn[p].y;
+  }
+}
+
 // One time step for all NS scenarios from the two words (w_v, w_x) of the step.
 // NS scenarios in registers; DYN: only the first L.n_scen of them are live.
 // Scenarios 1 .. NV differ from the base only in v0 (all constant deltas zero):
@@ -144,6 +238,10 @@ __device__ __forceinline__ void step_all(const PathLaunch& L, uint32_t w_v, uint
         c[s + 1] = cc.y;
       }
     }
+    return;
+  }
+  if constexpr (NS > 1 && !QEM && !DYN) {
+    step_merged<NS, NV>(L, xv, zv, zx, v, x, c);
     return;
   }
   step_scheme<(NS > 1), QEM>(L.sc[0], L.qm, xv, zv, zx, v[0], x[0], c[0]);
@@ -312,7 +410,7 @@ __device__ __forceinline__ void write_results(const PathLaunch& L, int k, const 
 // scenarios needs.
 template <int NS, bool QEM>
 constexpr int path_warps() {
-  return NS == 1 ? (QEM ? SIMR_QEM_WARPS : SIMR_PRICE_WARPS) : NS == 3 ? SIMR_FD3_WARPS : NS == 5 ? SIMR_FD5_WARPS : 16;
+  return NS == 1 ? (QEM ? SIMR_QEM_WARPS : SIMR_PRICE_WARPS) : NS == 3 ? SIMR_FD3_WARPS : NS == 5 ? SIMR_FD5_WARPS : SIMR_FD11_WARPS;
 }
 
 // Whether the kernel of NS scenarios has a loop for the step pairs' counter table:
