@@ -14,6 +14,7 @@
 // asset runs alone in scalar FP32.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "simr_device.cuh"
@@ -23,7 +24,14 @@
 namespace simr {
 namespace {
 
-constexpr int kBasketTpb = 256;
+// Warps per SM (one block): the register file split by the assets' states.
+#ifndef SIMR_BASKET8_WARPS
+#define SIMR_BASKET8_WARPS 20
+#endif
+template <int NA>
+constexpr int basket_warps() {
+  return NA == 2 ? 24 : NA == 4 ? 20 : NA == 8 ? SIMR_BASKET8_WARPS : 8;
+}
 
 // step_base<false> of two assets at once in packed FP32, lane for lane the
 // scalar step's operations and rounding.
@@ -87,12 +95,10 @@ __device__ __forceinline__ void step_pair_qem(const ScenConst2& c, const QemCons
   v = vn;
 }
 
-// One step of the asset pair (k, k + 1) from their variance uniforms (centred)
-// and spot uniforms' normals eps[0 .. k + 1]: z = Lc eps over the rows k, k + 1,
-// summed in column order as for one asset at a time.
-template <int NA, bool QEM>
-__device__ __forceinline__ void basket_pair_step(const BasketLaunch& L, const ScenConst2& c, int k, float2 xv,
-                                                 const float (&eps)[NA], float2& v, float2& x, float2& comp) {
+// The log-spot normal of the asset pair (k, k + 1): z = Lc eps over the rows k,
+// k + 1, summed in column order as for one asset at a time.
+template <int NA>
+__device__ __forceinline__ float2 basket_normal(const BasketLaunch& L, int k, const float (&eps)[NA]) {
   const float* ra = L.Lc + k * (k + 1) / 2;
   const float* rb = ra + k + 1;  // row k + 1
   float2 z = make_float2(0.0f, 0.0f);
@@ -102,7 +108,26 @@ __device__ __forceinline__ void basket_pair_step(const BasketLaunch& L, const Sc
     z = p_fma(make_float2(ra[j], rb[j]), p_bc(eps[j]), z);
   }
   z.y = __fmaf_rn(rb[k + 1], eps[k + 1], z.y);
-  const float2 zv = norminv_centered2(xv);
+  return z;
+}
+
+// One step of the asset pair (k, k + 1) from its words (variance words wv, spot
+// words wx): the two pairs of normals behind one test for tails, then the step.
+template <int NA, bool QEM>
+__device__ __forceinline__ void basket_pair_step(const BasketLaunch& L, int k, uint32_t wv0, uint32_t wv1,
+                                                 uint32_t wx0, uint32_t wx1, float (&eps)[NA], float2& v, float2& x,
+                                                 float2& comp) {
+  const ScenConst2& c = L.pk[k / 2];
+  const float2 xv = centered_uniform2(wv0, wv1), xx = centered_uniform2(wx0, wx1);
+  float2 zv, e, wcv, wcx;
+  const bool central = norminv_try2(xv, wcv, zv);
+  if (!(norminv_try2(xx, wcx, e) && central)) {
+    norminv_fix2(xv, wcv, zv);
+    norminv_fix2(xx, wcx, e);
+  }
+  eps[k] = e.x;
+  eps[k + 1] = e.y;
+  const float2 z = basket_normal<NA>(L, k, eps);
   if constexpr (QEM)
     step_pair_qem(c, L.qk[k / 2], xv, zv, z, v, x, comp);
   else
@@ -124,20 +149,83 @@ __device__ __forceinline__ void basket_lone_step(const BasketLaunch& L, int k, f
   step_scheme<false, QEM>(L.sc[k], L.qm[k], xv, norminv_centered(xv), z, v, x, comp);
 }
 
+// One path: sum_k w_k S0_k e^{x_k} at maturity.
+template <int NA, bool QEM>
+__device__ __forceinline__ float basket_path(const BasketLaunch& L, uint64_t path) {
+  const int na = L.n_assets;
+  const int kl = na - 1;  // the lone last asset when na is odd
+  const bool lone = na & 1;
+  const PhiloxLane pl = philox_lane(path, L.rk);  // shared by the assets' counters
+  float2 v[NA / 2], x[NA / 2], comp[NA / 2];  // the pairs
+  float eps[NA];
+  uint32_t wz[NA], ww[NA];  // the odd step's words of each asset
+  float vl = L.sc[kl].v0, xl = 0.0f, cl = 0.0f;  // the lone asset (odd counts)
+#pragma unroll
+  for (int q = 0; q < NA / 2; ++q) {
+    v[q] = make_float2(L.sc[2 * q].v0, L.sc[2 * q + 1].v0);
+    x[q] = make_float2(0.0f, 0.0f);
+    comp[q] = make_float2(0.0f, 0.0f);
+  }
+#pragma unroll 1
+  for (uint32_t p = 0; 2 * p < L.steps; ++p) {
+    // words 0, 1 drive the even step 2p, words 2, 3 the odd one
+#pragma unroll
+    for (int q = 0; q < NA / 2; ++q) {
+      const int k = 2 * q;
+      if (k + 1 >= na) break;
+      const uint4 wa = philox_draw(pl, philox_ctr(p, (uint32_t)k, L.rk), L.rk);
+      const uint4 wb = philox_draw(pl, philox_ctr(p, (uint32_t)(k + 1), L.rk), L.rk);
+      wz[k] = wa.z;
+      ww[k] = wa.w;
+      wz[k + 1] = wb.z;
+      ww[k + 1] = wb.w;
+      basket_pair_step<NA, QEM>(L, k, wa.x, wb.x, wa.y, wb.y, eps, v[q], x[q], comp[q]);
+    }
+    uint4 wl = make_uint4(0u, 0u, 0u, 0u);
+    if (lone) {
+      wl = philox_draw(pl, philox_ctr(p, (uint32_t)kl, L.rk), L.rk);
+      basket_lone_step<NA, QEM>(L, kl, centered_uniform(wl.x), eps, norminv_centered(centered_uniform(wl.y)), vl, xl, cl);
+    }
+    if (2 * p + 1 < L.steps) {
+#pragma unroll
+      for (int q = 0; q < NA / 2; ++q) {
+        const int k = 2 * q;
+        if (k + 1 >= na) break;
+        basket_pair_step<NA, QEM>(L, k, wz[k], wz[k + 1], ww[k], ww[k + 1], eps, v[q], x[q], comp[q]);
+      }
+      if (lone)
+        basket_lone_step<NA, QEM>(L, kl, centered_uniform(wl.z), eps, norminv_centered(centered_uniform(wl.w)), vl, xl,
+                                  cl);
+    }
+  }
+  float B = 0.0f;
+#pragma unroll
+  for (int q = 0; q < NA / 2; ++q) {
+    if (2 * q + 1 >= na) break;
+    B += terminal_spot(L.S0w[2 * q], x[q].x, comp[q].x);
+    B += terminal_spot(L.S0w[2 * q + 1], x[q].y, comp[q].y);
+  }
+  if (lone) B += terminal_spot(L.S0w[kl], xl, cl);
+  return B;
+}
+
+// One block per SM; its warps take 32-path batches item by item (ItemPlan), each
+// item's sums in the item's own row.  20 warps at 8 assets: 2,372 -> 2,170 us for
+// 252 steps x 2^18 paths x 32 strikes (16 warps 2,364: 54 batches a block; a
+// step-pair counter table per asset cost registers and made it 2,510).
 template <int NA, int TILE, bool QEM>
-__global__ void __launch_bounds__(kBasketTpb) heston_basket_kernel(const __grid_constant__ BasketLaunch L,
-                                                                   const double* __restrict__ strikes,
-                                                                   BasketOutputs out, double* __restrict__ partials,
-                                                                   unsigned int* __restrict__ ticket) {
+__global__ void __launch_bounds__(kWarp * basket_warps<NA>(), 1)
+    heston_basket_kernel(const __grid_constant__ BasketLaunch L, const __grid_constant__ ItemPlan I,
+                         const double* __restrict__ strikes, BasketOutputs out, double* __restrict__ partials,
+                         unsigned int* __restrict__ ticket) {
   static_assert(NA % 2 == 0, "assets are stepped in pairs");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warps = blockDim.x / kWarp;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int row = 2 * L.nk_pad;
-  double* acc = reinterpret_cast<double*>(smem_raw);
-  float* ks = reinterpret_cast<float*>(acc + (size_t)warps * row);
-  int* s_last = reinterpret_cast<int*>(ks + L.nk_pad);
-  for (int i = threadIdx.x; i < warps * row; i += blockDim.x) acc[i] = 0.0;
+  const int lane = threadIdx.x & 31;
+  int* s_flag = reinterpret_cast<int*>(smem_raw);
+  unsigned* s_next = reinterpret_cast<unsigned*>(s_flag + 1);
+  float* ks = reinterpret_cast<float*>(s_flag + 4);
+  const ItemRows rows(ks + ((L.nk_pad + 1) & ~1), I, 2 * L.nk_pad);
+  if (threadIdx.x == 0) *s_next = 0u;
   for (int j = threadIdx.x; j < L.nk_pad; j += blockDim.x) {
     float K = 0.0f;
     if (j < L.n_strikes) {
@@ -150,118 +238,50 @@ __global__ void __launch_bounds__(kBasketTpb) heston_basket_kernel(const __grid_
   __syncthreads();
 
   const bool put = L.is_put != 0;
-  const int na = L.n_assets;
-  const int kl = na - 1;  // the lone last asset when na is odd
-  double* my_acc = acc + (size_t)warp * row;
-  const uint64_t batches = (L.paths + kWarp - 1) / kWarp;
-  const uint64_t total_warps = (uint64_t)gridDim.x * warps;
-  for (uint64_t bt = (uint64_t)blockIdx.x * warps + warp; bt < batches; bt += total_warps) {
-    const uint64_t path = bt * kWarp + lane;
-    const bool active = path < L.paths;
-    const PhiloxLane pl = philox_lane(path, L.rk);  // shared by the assets' counters
-    float2 v[NA / 2], x[NA / 2], comp[NA / 2];  // the pairs
-    float eps[NA];
-    uint32_t wz[NA], ww[NA];  // the odd step's words of each asset
-    float vl = L.sc[kl].v0, xl = 0.0f, cl = 0.0f;  // the lone asset (odd counts)
-    uint32_t wzl = 0u, wwl = 0u;
-#pragma unroll
-    for (int q = 0; q < NA / 2; ++q) {
-      v[q] = make_float2(L.sc[2 * q].v0, L.sc[2 * q + 1].v0);
-      x[q] = make_float2(0.0f, 0.0f);
-      comp[q] = make_float2(0.0f, 0.0f);
-    }
-    for (uint32_t p = 0; 2 * p < L.steps; ++p) {
-      // even step 2p: draw each pair's words, correlate, step in pair order (an
-      // odd count's last asset alone)
-#pragma unroll
-      for (int q = 0; q < NA / 2; ++q) {
-        const int k = 2 * q;
-        if (k + 1 >= na) break;
-        const uint4 wa = philox_draw(pl, philox_ctr(p, (uint32_t)k, L.rk), L.rk);
-        const uint4 wb = philox_draw(pl, philox_ctr(p, (uint32_t)(k + 1), L.rk), L.rk);
-        wz[k] = wa.z;
-        ww[k] = wa.w;
-        wz[k + 1] = wb.z;
-        ww[k + 1] = wb.w;
-        const float2 e = norminv_centered2(centered_uniform2(wa.y, wb.y));
-        eps[k] = e.x;
-        eps[k + 1] = e.y;
-        basket_pair_step<NA, QEM>(L, L.pk[q], k, centered_uniform2(wa.x, wb.x), eps, v[q], x[q], comp[q]);
-      }
-      if (na & 1) {
-        const uint4 w = philox_draw(pl, philox_ctr(p, (uint32_t)kl, L.rk), L.rk);
-        wzl = w.z;
-        wwl = w.w;
-        basket_lone_step<NA, QEM>(L, kl, centered_uniform(w.x), eps, norminv_centered(centered_uniform(w.y)), vl, xl, cl);
-      }
-      if (2 * p + 1 < L.steps) {
-#pragma unroll
-        for (int q = 0; q < NA / 2; ++q) {
-          const int k = 2 * q;
-          if (k + 1 >= na) break;
-          const float2 e = norminv_centered2(centered_uniform2(ww[k], ww[k + 1]));
-          eps[k] = e.x;
-          eps[k + 1] = e.y;
-          basket_pair_step<NA, QEM>(L, L.pk[q], k, centered_uniform2(wz[k], wz[k + 1]), eps, v[q], x[q], comp[q]);
+  const uint64_t block0 = I.batches / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, I.batches % gridDim.x);
+  const uint64_t nb = I.batches / gridDim.x + (blockIdx.x < I.batches % gridDim.x ? 1 : 0);
+  while (true) {
+    unsigned it = 0;
+    if (lane == 0) it = atomicAdd(s_next, 1u);
+    it = __shfl_sync(kFull, it, 0);
+    uint64_t b0, b1;
+    if (!item_range(I, it, nb, b0, b1)) break;
+    ItemRow my = rows.at(I, it);
+    for (uint64_t b = b0; b < b1; ++b) {
+      const uint64_t path = (block0 + b) * kWarp + lane;
+      const bool active = path < L.paths;
+      const float B = basket_path<NA, QEM>(L, path);
+      if (TILE == 1) {
+        const float f = active ? (put ? fmaxf(ks[0] - B, 0.0f) : fmaxf(B - ks[0], 0.0f)) : 0.0f;
+        const float t0 = warp_sum(f), t1 = warp_sum(f * f);
+        if (lane == 0) {
+          my.add(0, t0);
+          my.add(1, t1);
         }
-        if (na & 1)
-          basket_lone_step<NA, QEM>(L, kl, centered_uniform(wzl), eps, norminv_centered(centered_uniform(wwl)), vl, xl,
-                               cl);
-      }
-    }
-    float B = 0.0f;  // sum_k w_k S0_k e^{x_k}
+      } else {
+        for (int t0 = 0; t0 < L.nk_pad; t0 += 32) {
+          float vf[32], vq[32];
 #pragma unroll
-    for (int q = 0; q < NA / 2; ++q) {
-      if (2 * q + 1 >= na) break;
-      B += terminal_spot(L.S0w[2 * q], x[q].x, comp[q].x);
-      B += terminal_spot(L.S0w[2 * q + 1], x[q].y, comp[q].y);
-    }
-    if (na & 1) B += terminal_spot(L.S0w[kl], xl, cl);
-
-    if (TILE == 1) {
-      const float f = active ? (put ? fmaxf(ks[0] - B, 0.0f) : fmaxf(B - ks[0], 0.0f)) : 0.0f;
-      const float t0 = warp_sum(f), t1 = warp_sum(f * f);
-      if (lane == 0) {
-        my_acc[0] += (double)t0;
-        my_acc[1] += (double)t1;
-      }
-    } else {
-      for (int t0 = 0; t0 < L.nk_pad; t0 += 32) {
-        float vf[32], vq[32];
-#pragma unroll
-        for (int jj = 0; jj < 32; ++jj) {
-          const float K = ks[t0 + jj];
-          const float f = active ? (put ? fmaxf(K - B, 0.0f) : fmaxf(B - K, 0.0f)) : 0.0f;
-          vf[jj] = f;
-          vq[jj] = f * f;
+          for (int jj = 0; jj < 32; ++jj) {
+            const float K = ks[t0 + jj];
+            const float f = active ? (put ? fmaxf(K - B, 0.0f) : fmaxf(B - K, 0.0f)) : 0.0f;
+            vf[jj] = f;
+            vq[jj] = f * f;
+          }
+          butterfly32(vf, lane);
+          butterfly32(vq, lane);
+          my.add(t0 + lane, vf[0]);
+          my.add(L.nk_pad + t0 + lane, vq[0]);
         }
-        butterfly32(vf, lane);
-        butterfly32(vq, lane);
-        my_acc[t0 + lane] += (double)vf[0];
-        my_acc[L.nk_pad + t0 + lane] += (double)vq[0];
       }
+      my.first = false;
     }
   }
   __syncthreads();
-
-  double* my_row = partials + (size_t)blockIdx.x * row;
-  for (int i = threadIdx.x; i < row; i += blockDim.x) {
-    double s = 0.0;
-    for (int w = 0; w < warps; ++w) s += acc[(size_t)w * row + i];
-    my_row[i] = s;
-  }
-  __threadfence();
+  sum_item_rows(rows, I, nb);
   __syncthreads();
-  if (threadIdx.x == 0) *s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1) ? 1 : 0;
-  __syncthreads();
-  if (!*s_last) return;
-  __threadfence();
-  for (int i = threadIdx.x; i < row; i += blockDim.x) {
-    double s = 0.0;
-    for (unsigned b = 0; b < gridDim.x; ++b) s += __ldcg(partials + (size_t)b * row + i);
-    acc[i] = s;
-  }
-  __syncthreads();
+  if (!sum_block_rows(rows.acc, rows.row, partials, ticket, s_flag)) return;
+  const double* acc = rows.acc;
   const double inv_n = 1.0 / L.paths_total;
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
   for (int k = threadIdx.x; k < L.n_strikes; k += blockDim.x) {
@@ -275,30 +295,23 @@ __global__ void __launch_bounds__(kBasketTpb) heston_basket_kernel(const __grid_
       out.stderr_[k] = bad ? nan : L.disc * sqrt(var > 0.0 ? var : 0.0);
     }
   }
-  if (threadIdx.x == 0) *ticket = 0u;
 }
 
 template <int NA, int TILE, bool QEM>
 cudaError_t launch_basket_t(const BasketLaunch& L, const double* strikes, const BasketOutputs& out,
                             double* partials, size_t partial_doubles, unsigned int* ticket, int num_sms,
                             cudaStream_t stream) {
-  const int warps = kBasketTpb / kWarp;
   const size_t row = 2 * (size_t)L.nk_pad;
-  const size_t smem = warps * row * sizeof(double) + L.nk_pad * sizeof(float) + 16;
+  const size_t head = 16 + ((L.nk_pad + 1) & ~1) * sizeof(float);
+  const uint64_t batches = (L.paths + kWarp - 1) / kWarp;
+  const uint64_t grid = std::min<uint64_t>(num_sms, batches);
+  const ItemPlan I = make_item_plan(batches, grid, basket_warps<NA>(), row, kItemBytes - head);
+  const size_t smem = head + item_rows_bytes(I, row);
   auto kern = heston_basket_kernel<NA, TILE, QEM>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBasketTpb, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const uint64_t batches = (L.paths + kWarp - 1) / kWarp;
-  uint64_t grid = (uint64_t)num_sms * per_sm;
-  const uint64_t need = (batches + warps - 1) / warps;
-  if (grid > need) grid = need;
-  if (grid < 1) grid = 1;
-  if ((size_t)grid * row > partial_doubles) return cudaErrorMemoryAllocation;
-  kern<<<(unsigned)grid, kBasketTpb, smem, stream>>>(L, strikes, out, partials, ticket);
+  if ((size_t)(grid + kRowGroups) * row > partial_doubles) return cudaErrorMemoryAllocation;
+  kern<<<(unsigned)grid, kWarp * I.warps, smem, stream>>>(L, I, strikes, out, partials, ticket);
   return cudaGetLastError();
 }
 
@@ -318,7 +331,7 @@ cudaError_t launch_basket_na(const BasketLaunch& L, const double* strikes, const
 }  // namespace
 
 size_t basket_partial_doubles(const BasketLaunch& L, int num_sms) {
-  return (size_t)num_sms * 8 * 2 * (size_t)L.nk_pad;  // at most 8 resident blocks per SM
+  return (size_t)(num_sms + kRowGroups) * 2 * (size_t)L.nk_pad;
 }
 
 cudaError_t launch_basket(const BasketLaunch& L, const double* strikes, const BasketOutputs& out, double* partials,
