@@ -85,7 +85,8 @@ __device__ __forceinline__ float lsm_payoff(bool put, float S, float K) {
 // Path kernel: states at the exercise dates, maturity cash flow.  One block per SM;
 // its warps take the block's 64-path batches from a counter in shared memory and
 // step two paths per thread through the pipelined loop.  Dynamic shared memory: the
-// step pairs' counter table (n_tab entries, 0: none).  252 dates x 2^20 paths.
+// step pairs' counter table (n_tab entries, 0: none).  Issue-bound like pricing; 252
+// dates x 2^20 paths: a valuation 3,543 -> 3,415 us (24 warps; 28 the same, 20 2% slower).
 template <bool QEM>
 __global__ void __launch_bounds__(kLsmPathTpb, 1) lsm_paths_kernel(const __grid_constant__ LsmLaunch L, int n_tab,
                                                                    float* __restrict__ S_out, float* __restrict__ V_out,
@@ -444,33 +445,39 @@ __global__ void __launch_bounds__(kLsmTpb) lsm_date_kernel(const __grid_constant
 // parts, then one refinement step whose residual b - G x is formed in
 // double-float (each product G x split exactly by an FMA).  The solution is the
 // pair (x, dx); x + dx in FP32 is what the exercise rule uses.
+// Every lane factors the whole matrix in its own registers: the same operations per
+// entry as one row per lane with shuffles between them (3,400 cycles a date), whose
+// exchanges were most of the chain; only the residual is one row per lane.
 __device__ void lsm_solve_df(const DF* tot, float* x_out, float* dx_out, int lane) {
+  constexpr int gi[kNB * kNB] = {0, 1, 3, 2,  4,  5,  1, 3,  6,  4,  7,  8,  3,  6,  10, 7,  11, 12,
+                                 2, 4, 7, 5,  8,  9,  4, 7,  11, 8,  12, 13, 5,  8,  12, 9,  13, 14};  // c_gram_index
   const int row = lane < kNB ? lane : 0;
-  DF g[kNB];
-  float l[kNB], rd[kNB];
-  unsigned keep = 0;
+  DF gr[kNB];  // this lane's row, for the residual
 #pragma unroll
-  for (int k = 0; k < kNB; ++k) {
-    g[k] = tot[c_gram_index[row * kNB + k]];
-    l[k] = 0.0f;
-  }
+  for (int k = 0; k < kNB; ++k) gr[k] = tot[c_gram_index[row * kNB + k]];
+  float g[kNMono], l[kNB][kNB], rd[kNB];
+#pragma unroll
+  for (int k = 0; k < kNMono; ++k) g[k] = tot[k].hi;
+  unsigned keep = 0;
 #pragma unroll
   for (int k = 0; k < kNB; ++k) {
     float s = 0.0f;
 #pragma unroll
-    for (int i = 0; i < k; ++i) s = fmaf(l[i], l[i], s);
-    const float d = __shfl_sync(kFull, g[k].hi - s, k);
-    const float gkk = __shfl_sync(kFull, g[k].hi, k);
-    rd[k] = 0.0f;
-    if (!(gkk > 0.0f && d > 1e-5f * gkk)) continue;
-    keep |= 1u << k;
-    const float lkk = __fsqrt_rn(d);
-    rd[k] = __frcp_rn(lkk);
-    float t = 0.0f;
+    for (int i = 0; i < k; ++i) s = fmaf(l[k][i], l[k][i], s);
+    const float gkk = g[gi[k * kNB + k]];
+    const float d = gkk - s;
+    const bool in = gkk > 0.0f && d > 1e-5f * gkk;
+    if (in) keep |= 1u << k;
+    const float lkk = in ? __fsqrt_rn(d) : 0.0f;
+    rd[k] = in ? __frcp_rn(lkk) : 0.0f;
+    l[k][k] = lkk;
 #pragma unroll
-    for (int i = 0; i < k; ++i) t = fmaf(l[i], __shfl_sync(kFull, l[i], k), t);
-    if (lane > k) l[k] = (g[k].hi - t) * rd[k];
-    if (lane == k) l[k] = lkk;
+    for (int r = k + 1; r < kNB; ++r) {
+      float t = 0.0f;
+#pragma unroll
+      for (int i = 0; i < k; ++i) t = fmaf(l[r][i], l[k][i], t);
+      l[r][k] = in ? (g[gi[r * kNB + k]] - t) * rd[k] : 0.0f;
+    }
   }
   auto solve = [&](const float (&r)[kNB], float (&x)[kNB]) {
     float z[kNB];
@@ -478,15 +485,14 @@ __device__ void lsm_solve_df(const DF* tot, float* x_out, float* dx_out, int lan
     for (int k = 0; k < kNB; ++k) {
       float t = 0.0f;
 #pragma unroll
-      for (int i = 0; i < k; ++i) t = fmaf(l[i], z[i], t);
-      const float zk = ((keep >> k) & 1u) ? (r[k] - t) * rd[k] : 0.0f;
-      z[k] = __shfl_sync(kFull, zk, k);
+      for (int i = 0; i < k; ++i) t = fmaf(l[k][i], z[i], t);
+      z[k] = ((keep >> k) & 1u) ? (r[k] - t) * rd[k] : 0.0f;
     }
 #pragma unroll
     for (int k = kNB - 1; k >= 0; --k) {
       float t = 0.0f;
 #pragma unroll
-      for (int i = k + 1; i < kNB; ++i) t = fmaf(__shfl_sync(kFull, l[k], i), x[i], t);
+      for (int i = k + 1; i < kNB; ++i) t = fmaf(l[i][k], x[i], t);
       x[k] = ((keep >> k) & 1u) ? (z[k] - t) * rd[k] : 0.0f;
     }
   };
@@ -497,9 +503,9 @@ __device__ void lsm_solve_df(const DF* tot, float* x_out, float* dx_out, int lan
   DF res = tot[kNMono + row];
 #pragma unroll
   for (int k = 0; k < kNB; ++k) {
-    const float p = g[k].hi * x[k];
-    const float pe = fmaf(g[k].hi, x[k], -p);  // exact remainder of the product
-    res = df_add(res, DF{-p, -fmaf(g[k].lo, x[k], pe)});
+    const float p = __fmul_rn(gr[k].hi, x[k]);
+    const float pe = fmaf(gr[k].hi, x[k], -p);  // exact remainder of the product
+    res = df_add(res, DF{-p, -fmaf(gr[k].lo, x[k], pe)});
   }
   const float r = res.hi + res.lo;
 #pragma unroll
@@ -567,7 +573,7 @@ __device__ __forceinline__ void bulk_copy_g2s(float* dst, const float* src, uint
 // Waits for the phase of the given parity to complete (non-blocking polls,
 // backing off like the grid barrier); false once the wait has expired.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  const unsigned long long t0 = global_ns();
+  unsigned long long t0 = 0;
   for (unsigned it = 1;; ++it) {
     uint32_t done;
     asm volatile(
@@ -576,6 +582,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
         : "r"(smem_addr(bar)), "r"(parity)
         : "memory");
     if (done) return true;
+    if (it == 1) t0 = global_ns();  // (not read when the copy has landed, the usual case)
     if (wait_expired(it, t0)) return false;
     if (it > 2048) __nanosleep(32);
   }
@@ -594,28 +601,33 @@ struct LsmSweep {
 // atomic and the polls.  Bounded: a wait that expires sets status bit 1 and
 // returns false, and every later barrier returns false at once, so all blocks
 // leave within one time-out.  `idle()` runs in every thread once the block has
-// arrived, while thread 0 waits.
+// arrived, while thread 0 waits.  The arrival is a release and the poll an acquire by
+// thread 0 alone (a fence in all 1,024 threads, and the status word read before the
+// arrival, put two round trips to L2 on every date's path).  With the solve above and
+// the timer read only by a wait that has to poll: 10.5 -> 9.8 us a date.
 template <class Idle>
 __device__ bool lsm_grid_sync(const LsmSweep& Y, unsigned nb, unsigned extra, int* s_flag, Idle&& idle) {
-  __threadfence();
   __syncthreads();
+  if (threadIdx.x == 0)  // (release: the block's row, ordered before by the barrier above)
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(Y.count), "r"(1u) : "memory");
   idle();
   if (threadIdx.x == 0) {
     int ok = (*(volatile int*)Y.status & 2) == 0;
     if (ok) {
       const unsigned target = (nb + 1u) * gridDim.x + extra;
-      atomicAdd(Y.count, 1u);
-      const unsigned long long t0 = global_ns();
-      unsigned it = 0;
-      while (*(volatile unsigned*)Y.count < target) {
-        if (wait_expired(++it, t0)) {
+      unsigned long long t0 = 0;
+      for (unsigned it = 1;; ++it) {
+        unsigned seen;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(Y.count) : "memory");
+        if (seen >= target) break;
+        if (it == 1) t0 = global_ns();
+        if (wait_expired(it, t0)) {
           atomicOr(Y.status, 2);
           ok = 0;
           break;
         }
         if (it > 2048) __nanosleep(32);
       }
-      __threadfence();
     }
     *s_flag = ok;
   }
@@ -699,6 +711,7 @@ __global__ void __launch_bounds__(kSweepTpb, 1) lsm_sweep_kernel(const __grid_co
   float2* beta_t = reinterpret_cast<float2*>(B.beta_t);  // [n_ex][6] (x, dx) pairs
   const uint64_t gt = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t g0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int live = g0 < P ? (int)min((uint64_t)M, (P - g0 + gt - 1) / gt) : 0;  // this thread's paths
   const bool put = L.is_put != 0;
   const float K = L.K;
   for (int k = threadIdx.x; k < L.n_ex; k += kSweepTpb) s_dpow[k] = B.dpow[k];
@@ -775,7 +788,7 @@ __global__ void __launch_bounds__(kSweepTpb, 1) lsm_sweep_kernel(const __grid_co
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         const float h = lsm_payoff(put, Su[m], K);
-        if (g0 + (uint64_t)m * gt < P && h > 0.0f &&
+        if (m < live && h > 0.0f &&
             h > lsm_continuation(bj, fmaf(Su[m], tj.x, tj.y), fmaf(Vu[m], tj.z, tj.w))) {
           s_c[m * kSweepTpb + threadIdx.x] = h;
           s_st[m * kSweepTpb + threadIdx.x] = d;
@@ -807,7 +820,7 @@ __global__ void __launch_bounds__(kSweepTpb, 1) lsm_sweep_kernel(const __grid_co
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         const float h = lsm_payoff(put, Sn[m], K);
-        if (g0 + (uint64_t)m * gt < P && h > 0.0f) {
+        if (m < live && h > 0.0f) {
           const int st = s_st[m * kSweepTpb + threadIdx.x];
           const float Yv = st >= 0 ? s_c[m * kSweepTpb + threadIdx.x] * s_dpow[st - (d - 1)] : 0.0f;
           lsm_accumulate(acc, fmaf(Sn[m], tr.x, tr.y), fmaf(Vn[m], tr.z, tr.w), Yv);
