@@ -34,10 +34,9 @@
 #include "simr_reduce.cuh"
 
 // Tuning knobs (compile-time): warps per SM.  Measured at 252 steps x 2^20 paths:
-// pricing 770 / 785 / 786 us at 24 / 28 / 32 warps (pipelined loop); 5 scenarios
-// 2,214 / 2,171 / 2,157 / 2,169 us at 20 / 24 / 28 / 32; 11 scenarios (365 x 250,001)
-// 1,707 / 1,728 / 1,918 us at 16 / 20 / 24; 3 scenarios (one strike, 64 x 65,536)
-// 41.6 / 42.2 / 42.4 us at 20 / 24 / 32.  QE-M pricing 285 / 289 / 242 us at 24 /
+// pricing 770 / 785 / 786 us at 24 / 28 / 32 warps (pipelined loops); 5 scenarios
+// 2,138 / 2,170 us at 24 / 28; 11 scenarios (365 x 250,001) 1,707 / 1,728 / 1,918 us at
+// 16 / 20 / 24; 3 scenarios (one strike, 64 x 65,536) 39 us at 20 and 24.  QE-M pricing 285 / 289 / 242 us at 24 /
 // 28 / 32 (101 x 300,007 x 40 strikes: 31 batches a block), before the pipelined loop.
 #ifndef SIMR_PRICE_WARPS
 #define SIMR_PRICE_WARPS 24
@@ -46,13 +45,13 @@
 #define SIMR_QEM_WARPS 32
 #endif
 #ifndef SIMR_FD3_WARPS
-#define SIMR_FD3_WARPS 24
+#define SIMR_FD3_WARPS 20
 #endif
 #ifndef SIMR_FD11_WARPS
 #define SIMR_FD11_WARPS 16
 #endif
 #ifndef SIMR_FD5_WARPS
-#define SIMR_FD5_WARPS 28
+#define SIMR_FD5_WARPS 24
 #endif
 // paths per thread of the pricing (one scenario) and bump-and-revalue kernels
 #ifndef SIMR_PRICE_PPT
@@ -128,9 +127,15 @@ __device__ __forceinline__ void pair_moments(const PathLaunch& L, int P, float2 
 // exponential branch, whose lanes are redone chain by chain.  (A test per chain kept
 // them apart: 252 steps x 2^20 paths x 32 strikes, 5 scenarios 2,230 -> 2,157 us; 11
 // scenarios at 365 x 250,001 x 21 1,806 -> 1,707.)
-template <int NS, int NV>
-__device__ __forceinline__ void step_merged(const PathLaunch& L, float xv, float zv, float zx, float (&v)[NS],
-                                            float (&x)[NS], float (&c)[NS]) {
+// d: the step's draws; with NEXT, on return the next step's, from its words,
+// computed beside the variance chains behind the same test.
+struct StepDraw {
+  float xv, zv, zx;  // 2 U_V - 1, Z_V, Z_X
+};
+template <int NS, int NV, bool NEXT>
+__device__ __forceinline__ void step_merged(const PathLaunch& L, StepDraw& d, uint32_t next_v, uint32_t next_x,
+                                            float (&v)[NS], float (&x)[NS], float (&c)[NS]) {
+  const float xv = d.xv, zv = d.zv, zx = d.zx;
   constexpr int NP = (NS - 1) / 2;
   const ScenConst& b = L.sc[0];
   const float m0 = __fadd_rn(__fmul_rn(v[0], b.E), b.thE);
@@ -146,7 +151,14 @@ __device__ __forceinline__ void step_merged(const PathLaunch& L, float xv, float
     pair_moments<NV>(L, p, make_float2(v[2 * p + 1], v[2 * p + 2]), m, s2h);
     quad &= qe_try2(m, s2h, p_bc(zv), m2, t, vn[p], dl[p]);
   }
-  if (!quad) {
+  float2 xu, wc, z;
+  bool central = true;
+  if constexpr (NEXT) {
+    xu = centered_uniform2(next_v, next_x);
+    central = norminv_try2(xu, wc, z);
+  }
+  if (!(quad && central)) {
+    if constexpr (NEXT) norminv_fix2(xu, wc, z);
     if (!(t0 > kQuadT)) qe_exp_branch(m0, s0, m20, xv, vn0, dl0);
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
@@ -196,6 +208,7 @@ __device__ __forceinline__ void step_merged(const PathLaunch& L, float xv, float
     v[2 * p + 1] = vn[p].x;
     v[2 * p + 2] = vn[p].y;
   }
+  if constexpr (NEXT) d = StepDraw{xu.x, z.x, z.y};
 }
 
 // One time step for all NS scenarios from the two words (w_v, w_x) of the step.
@@ -241,7 +254,8 @@ __device__ __forceinline__ void step_all(const PathLaunch& L, uint32_t w_v, uint
     return;
   }
   if constexpr (NS > 1 && !QEM && !DYN) {
-    step_merged<NS, NV>(L, xv, zv, zx, v, x, c);
+    StepDraw d{xv, zv, zx};
+    step_merged<NS, NV, false>(L, d, 0u, 0u, v, x, c);
     return;
   }
   step_scheme<(NS > 1), QEM>(L.sc[0], L.qm, xv, zv, zx, v[0], x[0], c[0]);
@@ -294,12 +308,9 @@ __device__ __forceinline__ void step_paths(const PathLaunch& L, const uint32_t (
 // on the host in FP64, where M exists at every scenario's v0), v' has no term of
 // its own and dl the coefficient K2.
 template <int NS, bool DYN, bool QEM = false>
-__device__ __forceinline__ void step0_all(const PathLaunch& L, uint32_t w_v, uint32_t w_x, float (&v)[NS],
-                                          float (&x)[NS], float (&c)[NS]) {
-  const float xv = centered_uniform(w_v);
+__device__ __forceinline__ void step0_apply(const PathLaunch& L, float xv, float zv, float zx, float (&v)[NS],
+                                            float (&x)[NS], float (&c)[NS]) {
   const float omu = one_minus_u(xv);
-  const float zv = norminv_centered(xv);
-  const float zx = norminv_centered(centered_uniform(w_x));
   const ScenConst zero{};
   FirstConst fz = L.f0[0];
   fz.a = fz.b = fz.C = fz.L = fz.m0 = fz.K0p = 0.0f;  // base: zero deltas, its own threshold
@@ -318,6 +329,60 @@ __device__ __forceinline__ void step0_all(const PathLaunch& L, uint32_t w_v, uin
     }
     step0_crn(L.f0[0], s == 0 ? fz : L.f0[s], b0, d0, L.sc[s].v0, omu, zv, zx, v[s], x[s], c[s]);
   }
+}
+
+template <int NS, bool DYN, bool QEM = false>
+__device__ __forceinline__ void step0_all(const PathLaunch& L, uint32_t w_v, uint32_t w_x, float (&v)[NS],
+                                          float (&x)[NS], float (&c)[NS]) {
+  const float xv = centered_uniform(w_v);
+  step0_apply<NS, DYN, QEM>(L, xv, norminv_centered(xv), norminv_centered(centered_uniform(w_x)), v, x, c);
+}
+
+// One path of a 3- or 5-scenario launch under QE, software-pipelined: while a step's
+// chains run, the next step's normals and the next pair's Philox rounds are
+// computed (one strike, 64 x 65,536, 3 scenarios 41.0 -> 39.0 us; 5 scenarios at 100 x
+// 20,000 73.9 -> 67.7, at 252 x 2^20 2,157 -> 2,138; with 11 scenarios, whose chains
+// fill the issue by themselves, it was 7% slower).
+template <bool TAB, int NS, int NV>
+__device__ __forceinline__ void simulate_fd(const PathLaunch& L, const uint4* tab, uint64_t path, float (&v)[NS],
+                                            float (&x)[NS], float (&c)[NS]) {
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    v[s] = L.sc[s].v0;
+    x[s] = 0.0f;
+    c[s] = 0.0f;
+  }
+  const PhiloxLane pl[1] = {philox_lane(path, L.rk)};
+  uint4 w[1], n[1];
+  philox_draws<TAB, 1>(tab, 0u, L.option_index, L.rk, pl, w);
+  StepDraw d;
+  {
+    const float2 xu = centered_uniform2(w[0].x, w[0].y);
+    const float2 z = norminv_centered2(xu);
+    d = StepDraw{xu.x, z.x, z.y};
+  }
+  const uint32_t pairs = L.steps >> 1;
+  uint32_t i = 0;
+  if (L.first_split) {  // step 0 of every scenario from its own constants, then step 1
+    step0_apply<NS, false>(L, d.xv, d.zv, d.zx, v, x, c);
+    if (pairs) {
+      const float2 xu = centered_uniform2(w[0].z, w[0].w);
+      const float2 z = norminv_centered2(xu);
+      d = StepDraw{xu.x, z.x, z.y};
+      philox_draws<TAB, 1>(tab, 1u, L.option_index, L.rk, pl, w);
+      step_merged<NS, NV, true>(L, d, w[0].x, w[0].y, v, x, c);
+    }
+    i = 1;
+  }
+#pragma unroll 1
+  for (; i < pairs; ++i) {
+    philox_draws<TAB, 1>(tab, i + 1, L.option_index, L.rk, pl, n);  // (one pair past the last step is not used)
+    step_merged<NS, NV, true>(L, d, w[0].z, w[0].w, v, x, c);
+    step_merged<NS, NV, true>(L, d, n[0].x, n[0].y, v, x, c);
+    w[0] = n[0];
+  }
+  if ((L.steps & 1u) && !(L.first_split && L.steps == 1))  // odd last step
+    step_merged<NS, NV, true>(L, d, 0u, 0u, v, x, c);
 }
 
 // PPT paths per thread, simulated step by step in lockstep: independent
@@ -486,6 +551,11 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
         x[1][0] = x2.y;
         c[0][0] = c2.x;
         c[1][0] = c2.y;
+      } else if constexpr ((NS == 3 || NS == 5) && PPT == 1 && !QEM && !DYN) {
+        if (USE_TAB && tab)
+          simulate_fd<USE_TAB, NS, NV>(L, tab, pth[0], v[0], x[0], c[0]);
+        else
+          simulate_fd<false, NS, NV>(L, nullptr, pth[0], v[0], x[0], c[0]);
       } else if (USE_TAB && tab) {
         simulate_ppt<USE_TAB, NS, NV, DYN, PPT, QEM>(L, tab, pth, v, x, c);
       } else {
@@ -579,7 +649,9 @@ cudaError_t launch_t(const PathLaunch& L0, const double* strikes, const PathOutp
   const int tpb = kWarp * I.warps;
   const size_t smem = head + item_rows_bytes(I, row);
   auto kern = heston_paths_kernel<NS, NV, TILE, DYN, PPT, QEM>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024)  // (below, the default suffices)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if ((size_t)(grid + kRowGroups) * row > s.partial_doubles) return cudaErrorMemoryAllocation;
   *grid_used = (int)grid;
