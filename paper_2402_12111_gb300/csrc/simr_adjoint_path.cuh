@@ -515,11 +515,11 @@ __device__ __forceinline__ void keep_step_pipe(const ScenConst& c, const PairDra
   }
   v = vn;
 }
-// The odd step of a pair.
-__device__ __forceinline__ void keep_step_odd(const ScenConst& c, const PairDraw& d, float2& vd, float& v) {
+// One step alone.
+__device__ __forceinline__ void keep_step(const ScenConst& c, float xv, float zv, float2& vd, float& v) {
   float vn;
-  const KeepStep k = keep_try(c, v, d.zv.y, vd, vn);
-  if (!k.quad) keep_fix(k, d.xv.y, vd, vn);
+  const KeepStep k = keep_try(c, v, zv, vd, vn);
+  if (!k.quad) keep_fix(k, xv, vd, vn);
   v = vn;
 }
 
@@ -604,18 +604,26 @@ __device__ __forceinline__ void path_sweep(const ScenConst& c, const AdjConst& A
       float2 xx, wcv, wcx;
       if (!pair_draw_try(w[0], d, xx, wcv, wcx)) pair_draw_fix(d, xx, wcv, wcx);
     }
+    // (the last pair draws no next one: a checkpoint every 16 / 32 steps 2.44 -> 2.37 / 9.7 -> 9.2 ms,
+    // 252 / 1,024 steps x 2^20 paths)
+    const uint32_t last = (n1 - 1) / 2;
+    float2 vd;
 #pragma unroll 1
-    for (uint32_t p = n0 / 2; 2 * p < n1; ++p, wp += r3) {
-      philox_draws<TAB, 1>(tab, p + 1, option, rk, pl, w);  // (the pair past the segment is drawn and not used)
-      float2 vd;
+    for (uint32_t p = n0 / 2; p < last; ++p, wp += r3) {
+      philox_draws<TAB, 1>(tab, p + 1, option, rk, pl, w);
       keep_step_pipe(c, d, w[0], dn, vd, vv);
       wp[0] = vd;
       wp[r2] = d.zx;
-      if (2 * p + 1 < n1) {
-        keep_step_odd(c, d, vd, vv);
-        wp[r1] = vd;
-      }
+      keep_step(c, d.xv.y, d.zv.y, vd, vv);
+      wp[r1] = vd;
       d = dn;
+    }
+    keep_step(c, d.xv.x, d.zv.x, vd, vv);
+    wp[0] = vd;
+    wp[r2] = d.zx;
+    if (2 * last + 1 < n1) {
+      keep_step(c, d.xv.y, d.zv.y, vd, vv);
+      wp[r1] = vd;
     }
     float vnext = vv;  // v_{n1}
     // the reverse steps, from the top pair down
