@@ -276,31 +276,12 @@ __device__ __forceinline__ void step_all(const PathLaunch& L, uint32_t w_v, uint
   }
 }
 
-// One time step of PPT paths.  Pricing with two paths per thread runs the two
-// paths' steps paired (their inverse normals too; QE or QE-M); otherwise
-// step_all per path.
+// One time step of PPT paths, path by path.
 template <int NS, int NV, bool DYN, int PPT, bool QEM>
 __device__ __forceinline__ void step_paths(const PathLaunch& L, const uint32_t (&wv)[PPT], const uint32_t (&wx)[PPT],
                                            float (&v)[PPT][NS], float (&x)[PPT][NS], float (&c)[PPT][NS]) {
-  if constexpr (NS == 1 && PPT == 2) {
-    const float2 xv = centered_uniform2(wv[0], wv[1]);
-    const float2 zv = norminv_centered2(xv);
-    const float2 zx = norminv_centered2(centered_uniform2(wx[0], wx[1]));
-    float2 vv = make_float2(v[0][0], v[1][0]), xx = make_float2(x[0][0], x[1][0]), cc = make_float2(c[0][0], c[1][0]);
-    if constexpr (QEM)
-      step_qem2(L.sc[0], L.qm, xv, zv, zx, vv, xx, cc);
-    else
-      step_base2<false>(L.sc[0], xv, zv, zx, vv, xx, cc);
-    v[0][0] = vv.x;
-    v[1][0] = vv.y;
-    x[0][0] = xx.x;
-    x[1][0] = xx.y;
-    c[0][0] = cc.x;
-    c[1][0] = cc.y;
-  } else {
 #pragma unroll
-    for (int j = 0; j < PPT; ++j) step_all<NS, NV, DYN, QEM>(L, wv[j], wx[j], v[j], x[j], c[j]);
-  }
+  for (int j = 0; j < PPT; ++j) step_all<NS, NV, DYN, QEM>(L, wv[j], wx[j], v[j], x[j], c[j]);
 }
 
 // Step 0 of every scenario of a common-random-number launch (see step0_crn).
