@@ -345,7 +345,7 @@ cudaError_t launch_adjoint_t(const PathLaunch& L, const AdjConst& A, const doubl
   const size_t row = (size_t)kAdjAcc * L.nk_pad;
   const size_t smem = adjoint_smem_bytes_t(L, A, tpb, PPT, RACC);
   auto kern = heston_adjoint_kernel<TILE, PPT, RACC, QEM>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tpb, smem);
@@ -388,7 +388,7 @@ cudaError_t launch_adjoint_seg(const PathLaunch& L0, const AdjConst& A, const do
   const int tpb = kWarp * h.I.warps;
   const size_t row = (size_t)kAdjAcc * L.nk_pad;
   auto kern = heston_adjoint_seg_kernel<TILE, QEM>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem);
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   if ((size_t)(h.grid + kRowGroups) * row > s.partial_doubles) return cudaErrorMemoryAllocation;
   if ((size_t)h.grid * tpb * adjoint_ckpt_floats(A, 1) > s.ckpt_floats) return cudaErrorMemoryAllocation;
@@ -436,7 +436,7 @@ cudaError_t adjoint_max_ckpt_every(const PathLaunch& L, int steps_cap, int* k_ma
     const size_t smem = adjoint_smem_bytes_t(L, A, 128, SIMR_ADJ_PPT, racc);
     *n = 0;
     if (smem > kAdjMaxSmem) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kern, 128, smem);
   };
@@ -477,7 +477,7 @@ cudaError_t launch_paths_adjoint(const PathLaunch& L, const AdjConst& A, float* 
   const int tpb = 128;
   const size_t smem = (size_t)adjoint_thread_floats(A.n_seg, A.ckpt_every, 1) * tpb * sizeof(float);
   auto kern = L.scheme == 1 ? heston_paths_adjoint_kernel<true> : heston_paths_adjoint_kernel<false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   const uint64_t grid = (L.path_count + tpb - 1) / tpb;
   kern<<<(unsigned)grid, tpb, smem, stream>>>(L, A, x_T, grad);

@@ -1632,7 +1632,7 @@ int simr_lsm_price(simr_ctx* ctx, const simr_heston* model, double K, int is_put
   if (exercise_every < 1 || steps % exercise_every != 0)
     return fail(SIMR_EINVAL, "exercise_every must be >= 1 and divide steps");
   const uint32_t n_ex = steps / exercise_every;
-  if (n_ex > 8192) return fail(SIMR_EINVAL, "at most 8192 exercise dates");
+  if (n_ex > kLsmMaxDates) return fail(SIMR_EINVAL, "at most %u exercise dates", kLsmMaxDates);
   if (paths < 2 || paths > (1ull << 31)) return fail(SIMR_EINVAL, "paths must lie in [2, 2^31]");
   if ((double)n_ex * (double)paths * 8.0 > 64.0 * (1ull << 30))
     return fail(SIMR_EUNSUPPORTED, "the states at the exercise dates would exceed 64 GiB");

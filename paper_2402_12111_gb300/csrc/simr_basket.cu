@@ -308,7 +308,7 @@ cudaError_t launch_basket_t(const BasketLaunch& L, const double* strikes, const 
   const ItemPlan I = make_item_plan(batches, grid, basket_warps<NA>(), row, kItemBytes - head);
   const size_t smem = head + item_rows_bytes(I, row);
   auto kern = heston_basket_kernel<NA, TILE, QEM>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   if ((size_t)(grid + kRowGroups) * row > partial_doubles) return cudaErrorMemoryAllocation;
   kern<<<(unsigned)grid, kWarp * I.warps, smem, stream>>>(L, I, strikes, out, partials, ticket);

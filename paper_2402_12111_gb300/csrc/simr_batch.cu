@@ -223,7 +223,7 @@ void batch_variant(int v, bool adjoint, BatchLaunch* B) {
 }
 
 cudaError_t prepare_batch(const BatchLaunch& B) {
-  return cudaFuncSetAttribute(batch_kernel(B), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem(B));
+  return allow_dynamic_smem(batch_kernel(B));
 }
 
 cudaError_t batch_gseg_threads(int num_sms, size_t* threads) {

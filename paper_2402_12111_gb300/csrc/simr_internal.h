@@ -165,6 +165,17 @@ inline size_t item_rows_bytes(const ItemPlan& I, size_t row) {
 }
 // Dynamic shared memory a path kernel's block may take for them.
 constexpr size_t kItemBytes = 208 * 1024;
+
+// Dynamic shared memory a block may have at most (without static).
+constexpr size_t kMaxDynamicSmem = 227 * 1024;
+// Lifts `kern`'s limit on dynamic shared memory to `cap`.  The limit belongs to the
+// kernel, for every host thread and context on the device: it is always set to the
+// kernel's one cap and never to a call's own size, which a call on another thread
+// could lower between here and the launch.
+template <class Kernel>
+cudaError_t allow_dynamic_smem(Kernel kern, size_t cap = kMaxDynamicSmem) {
+  return cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
+}
 // Entries of the shared-memory table of step-pair counters for L's paths and steps.
 struct PathLaunch;
 int pair_table_entries(const PathLaunch& L);
@@ -239,6 +250,7 @@ cudaError_t launch_normals(const uint32_t* words, uint64_t n, float* z, float* z
 
 // Longstaff-Schwartz (simr_lsm.cu).  Exercise dates t_j = (j + 1) every dt,
 // j = 0 .. n_ex - 1; per-path states at the dates in [date][path] arrays.
+constexpr uint32_t kLsmMaxDates = 8192;
 struct LsmLaunch {
   uint32_t rk[10][2];
   ScenConst sc;        // base scenario constants (v0 included)

@@ -930,7 +930,8 @@ cudaError_t try_sweep_m(const LsmLaunch& L, const LsmBuffers& B, const LsmSweep&
   // S and v (two buffers), cash flow, exercise date; the discount table
   const size_t smem = ((size_t)6 * M * kSweepTpb + (size_t)L.n_ex) * sizeof(float);
   auto kern = lsm_sweep_kernel<M>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the kernel has static shared memory too: its cap is its largest call's)
+  cudaError_t e = allow_dynamic_smem(kern, ((size_t)6 * M * kSweepTpb + kLsmMaxDates) * sizeof(float));
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSweepTpb, smem);

@@ -632,7 +632,7 @@ cudaError_t launch_t(const PathLaunch& L0, const double* strikes, const PathOutp
   auto kern = heston_paths_kernel<NS, NV, TILE, DYN, PPT, QEM>;
   cudaError_t e = cudaSuccess;
   if (smem > 48 * 1024)  // (below, the default suffices)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   if ((size_t)(grid + kRowGroups) * row > s.partial_doubles) return cudaErrorMemoryAllocation;
   *grid_used = (int)grid;
