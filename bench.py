@@ -111,7 +111,7 @@ def measured_peaks():
 # The sources the bench step's kernel (heston_paths_kernel) is compiled from.
 PATH_KERNEL_SOURCES = ("paper_2402_12111_gb300/csrc/simr_paths.cu", "paper_2402_12111_gb300/csrc/simr_device.cuh",
                        "paper_2402_12111_gb300/csrc/simr_reduce.cuh", "paper_2402_12111_gb300/csrc/simr_internal.h",
-                       "include/simr.h")
+                       "paper_2402_12111_gb300/csrc/simr_items.h", "include/simr.h")
 
 
 def _code_only(text: str) -> str:

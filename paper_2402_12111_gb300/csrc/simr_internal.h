@@ -7,6 +7,7 @@
 
 #include "simr.h"
 #include "simr_device.cuh"
+#include "simr_items.h"
 
 namespace simr {
 
@@ -138,33 +139,6 @@ struct BatchOutputs {
   double* stderr_;  // [n_opts] or null
   double* grad;     // [n_opts][7] or null
 };
-
-// How the blocks of a path kernel hand their batches (a warp's paths of one pass)
-// to their warps.  Block b owns a contiguous run of the launch's batches, cut into
-// items by this plan alone: `levels` levels of one item per warp, each level three
-// fifths of what is left, then items of tail_size batches.  A warp takes the next
-// item from a counter in shared memory and leaves the item's sums in the item's
-// own row (FP64; FP32 for an item of one batch, whose sums are FP32), so the
-// totals do not depend on which warp took what.
-constexpr int kItemLevels = 12;
-struct ItemPlan {
-  uint64_t batches;               // of the whole launch
-  uint64_t size[kItemLevels];     // batches per item of a level
-  uint64_t begin[kItemLevels];    // the level's first batch within the block
-  uint64_t tail_begin, tail_size;
-  int32_t levels, warps;          // items per level = warps per block
-  int32_t rows64, rows32;         // most FP64 and FP32 rows a block uses
-};
-// The plan of `batches` on a grid of blocks of at most max_warps warps, with rows
-// of `row` sums in `bytes` of shared memory (at least one FP64 row).
-ItemPlan make_item_plan(uint64_t batches, uint64_t grid, int max_warps, size_t row, size_t bytes);
-// Shared memory of a plan's rows and of the block's totals behind them.
-inline size_t item_rows_bytes(const ItemPlan& I, size_t row) {
-  const size_t wide = row > 32u * I.warps ? row : 32u * I.warps;  // sum_item_rows' columns side by side
-  return (I.rows64 + 0ull) * row * 8 + wide * 8 + (I.rows32 * row + 1) / 2 * 8;
-}
-// Dynamic shared memory a path kernel's block may take for them.
-constexpr size_t kItemBytes = 208 * 1024;
 
 // Dynamic shared memory a block may have at most (without static).
 constexpr size_t kMaxDynamicSmem = 227 * 1024;

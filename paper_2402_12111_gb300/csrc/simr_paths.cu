@@ -652,43 +652,6 @@ int pair_table_entries(const PathLaunch& L) {
   return one_high_word && n <= 2048 ? (int)n : 0;
 }
 
-ItemPlan make_item_plan(uint64_t batches, uint64_t grid, int max_warps, size_t row, size_t bytes) {
-  ItemPlan I{};
-  I.batches = batches;
-  const uint64_t q = batches / grid, most = (batches + grid - 1) / grid;  // batches of a block
-  const uint64_t fits = (bytes - row * 8) / (row * 8);                    // FP64 rows beside the totals
-  uint64_t w = std::max<uint64_t>(1, std::min<uint64_t>({(uint64_t)max_warps, fits, most}));
-  // few batches a warp: as many warps as make the rounds even (31 batches on 28
-  // warps: two rounds of 16, not 28 and 3)
-  const uint64_t rounds = (most + w - 1) / w;
-  if (rounds == 2) w = (most + rounds - 1) / rounds;
-  I.warps = (int)w;
-  bytes -= std::max<size_t>(row, 32 * w) * 8 + 8;
-  // the fewest levels after which the rest, batch by batch in FP32 rows, fits; if
-  // none does, levels as long as the rows leave three wider FP64 items a warp
-  uint64_t rem = q;
-  while ((uint64_t)I.levels * w * row * 8 + (rem + 1) * row * 4 > bytes && I.levels < kItemLevels &&
-         rem * 3 >= 5 * w && (uint64_t)(I.levels + 4) * w * row * 8 <= bytes) {
-    const uint64_t size = rem * 3 / (5 * w);
-    I.size[I.levels] = size;
-    I.begin[I.levels] = q - rem;
-    ++I.levels;
-    rem -= size * w;
-  }
-  const uint64_t left = rem + (most - q), used = (uint64_t)I.levels * w;
-  I.tail_begin = q - rem;
-  I.tail_size = 1;
-  I.rows64 = (int32_t)used;
-  I.rows32 = (int32_t)left;
-  if ((used * 8 + left * 4) * row > bytes) {
-    const uint64_t room = bytes / (row * 8) - used;
-    I.tail_size = std::max<uint64_t>(2, (left + room - 1) / room);
-    I.rows64 = (int32_t)(used + (left + I.tail_size - 1) / I.tail_size);
-    I.rows32 = 0;
-  }
-  return I;
-}
-
 size_t paths_scratch_doubles(const PathLaunch& L, int num_sms) {
   return (size_t)(num_sms + kRowGroups) * (size_t)L.n_acc * L.nk_pad;
 }

@@ -33,20 +33,6 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// The batches [b0, b1) of item `it` of a block that owns nb batches; false past the last.
-__device__ __forceinline__ bool item_range(const ItemPlan& I, uint32_t it, uint64_t nb, uint64_t& b0, uint64_t& b1) {
-  const uint32_t lvl = it / (uint32_t)I.warps;
-  if (lvl < (uint32_t)I.levels) {
-    b0 = I.begin[lvl] + (uint64_t)(it - lvl * I.warps) * I.size[lvl];
-    b1 = b0 + I.size[lvl];
-  } else {
-    b0 = I.tail_begin + (uint64_t)(it - (uint32_t)(I.levels * I.warps)) * I.tail_size;
-    b1 = b0 + I.tail_size;
-  }
-  if (b1 > nb) b1 = nb;
-  return b0 < nb;
-}
-
 // An item's row: the sums of its batches, added in FP64 in batch order -- or, for
 // an item of one batch, that batch's FP32 sums as they are.
 struct ItemRow {
