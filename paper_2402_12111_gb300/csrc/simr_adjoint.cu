@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kWarp * (QEM ? SIMR_ADJ_QEM_WARPS : SIMR_ADJ_W
   int* s_flag = reinterpret_cast<int*>(ks + L.nk_pad);
   unsigned* s_next = reinterpret_cast<unsigned*>(s_flag + 1);
   uint4* tab = L.pair_table ? reinterpret_cast<uint4*>(s_flag + 4) : nullptr;
-  const ItemRows rows(s_flag + 4 + 4 * L.pair_table, I, kAdjAcc * L.nk_pad);
+  const ItemRows rows{smem_raw, (unsigned)(L.nk_pad * sizeof(StrikeConst) + 16 + L.pair_table * sizeof(uint4)), kAdjAcc * L.nk_pad};
   // checkpoints: this thread's column of a [slot][grid threads] global array
   float* ck = gckpt + (int)blockIdx.x * bd + tid;
   const int ck_stride = (int)(gridDim.x * blockDim.x);
@@ -297,25 +297,25 @@ __global__ void __launch_bounds__(kWarp * (QEM ? SIMR_ADJ_QEM_WARPS : SIMR_ADJ_W
       if (TILE == 1) {
         for (int a = 0; a < kAdjAcc; ++a) {
           const float t = warp_sum(act[0] ? adj_term(a, put, S[0], ks[0].K, g[0], A.invS0, A.T) : 0.0f);
-          if (lane == 0) my.add(a, t);
+          if (lane == 0) my.add<false>(smem_raw, a, t);
         }
       } else {
         for (int t0 = 0; t0 < L.nk_pad; t0 += 32) {
           float t[kAdjAcc];
           strike_tile_terms<1>(put, ks[t0 + lane].K, S, act, g, t);
 #pragma unroll
-          for (int a = 0; a < kAdjAcc; ++a) my.add(a * L.nk_pad + t0 + lane, t[a]);
+          for (int a = 0; a < kAdjAcc; ++a) my.add<false>(smem_raw, a * L.nk_pad + t0 + lane, t[a]);
         }
       }
-      my.first = false;
+      my.next_batch();
     }
   }
   __syncthreads();
   sum_item_rows(rows, I, nb);
   __syncthreads();
-  if (!sum_block_rows(rows.acc, rows.row, partials, ticket, s_flag)) return;
+  if (!sum_block_rows(rows.acc(I), rows.row, partials, ticket, s_flag)) return;
   // (a tile's third sum holds the weights w: the S0 column is w / S0)
-  write_adjoint(L, A, strikes, rows.acc, TILE == 1 ? 1.0 : (double)A.invS0, out);
+  write_adjoint(L, A, strikes, rows.acc(I), TILE == 1 ? 1.0 : (double)A.invS0, out);
 }
 
 // Per-path output: x_T and g = d x_T / d(v0, kappa, theta, sigma, rho).

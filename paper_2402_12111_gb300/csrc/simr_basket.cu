@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kWarp * basket_warps<NA>(), 1)
   int* s_flag = reinterpret_cast<int*>(smem_raw);
   unsigned* s_next = reinterpret_cast<unsigned*>(s_flag + 1);
   float* ks = reinterpret_cast<float*>(s_flag + 4);
-  const ItemRows rows(ks + ((L.nk_pad + 1) & ~1), I, 2 * L.nk_pad);
+  const ItemRows rows{smem_raw, (unsigned)(16 + ((L.nk_pad + 1) & ~1) * sizeof(float)), 2 * L.nk_pad};
   if (threadIdx.x == 0) *s_next = 0u;
   for (int j = threadIdx.x; j < L.nk_pad; j += blockDim.x) {
     float K = 0.0f;
@@ -255,8 +255,8 @@ __global__ void __launch_bounds__(kWarp * basket_warps<NA>(), 1)
         const float f = active ? (put ? fmaxf(ks[0] - B, 0.0f) : fmaxf(B - ks[0], 0.0f)) : 0.0f;
         const float t0 = warp_sum(f), t1 = warp_sum(f * f);
         if (lane == 0) {
-          my.add(0, t0);
-          my.add(1, t1);
+          my.add<false>(smem_raw, 0, t0);
+          my.add<false>(smem_raw, 1, t1);
         }
       } else {
         for (int t0 = 0; t0 < L.nk_pad; t0 += 32) {
@@ -270,18 +270,18 @@ __global__ void __launch_bounds__(kWarp * basket_warps<NA>(), 1)
           }
           butterfly32(vf, lane);
           butterfly32(vq, lane);
-          my.add(t0 + lane, vf[0]);
-          my.add(L.nk_pad + t0 + lane, vq[0]);
+          my.add<false>(smem_raw, t0 + lane, vf[0]);
+          my.add<false>(smem_raw, L.nk_pad + t0 + lane, vq[0]);
         }
       }
-      my.first = false;
+      my.next_batch();
     }
   }
   __syncthreads();
   sum_item_rows(rows, I, nb);
   __syncthreads();
-  if (!sum_block_rows(rows.acc, rows.row, partials, ticket, s_flag)) return;
-  const double* acc = rows.acc;
+  if (!sum_block_rows(rows.acc(I), rows.row, partials, ticket, s_flag)) return;
+  const double* acc = rows.acc(I);
   const double inv_n = 1.0 / L.paths_total;
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
   for (int k = threadIdx.x; k < L.n_strikes; k += blockDim.x) {

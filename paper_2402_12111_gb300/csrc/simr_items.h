@@ -86,23 +86,23 @@ inline ItemPlan make_item_plan(uint64_t batches, uint64_t grid, int max_warps, s
   I.rows64 = (int32_t)used;
   I.rows32 = (int32_t)left;
   if ((used * 8 + left * 4) * row > bytes) {
-    // wider items, in FP64 rows: whole rounds of one item a warp -- as many of them as
-    // the rows leave room for, or fewer where the warps then end by more than an eighth
-    // earlier.  (Cut by the rows alone they can leave a last round for a few warps: 5
+    // wider items, in FP64 rows: as many as the rows leave room for or whole rounds of
+    // one item a warp, whichever lets the warps end first (the more items of those within
+    // a sixteenth).  Cut by the rows alone they can leave a last round for a few warps: 5
     // scenarios x 128 strikes at 100 steps x 2^19 paths had 27 items of 4 batches on 24
-    // warps, 1,211 us against 977.)
-    const uint64_t room = bytes / (row * 8) - used;
-    const auto size = [&](uint64_t r) {
-      const uint64_t n = std::min(room, r * w);
+    // warps, 1,211 us against 977.
+    const uint64_t room = bytes / (row * 8) - used, all = room / w;
+    const auto size = [&](uint64_t r) {  // r rounds; past the last: as many items as rows
+      const uint64_t n = r > all ? room : std::min(room, std::max<uint64_t>(1, r) * w);
       return std::max<uint64_t>(2, (left + n - 1) / n);
     };
     const auto end = [&](uint64_t r) {  // batches of the warp with most of them
-      const uint64_t n = (left + size(r) - 1) / size(r);
-      return (n + w - 1) / w * size(r);
+      const uint64_t full = left / size(r), part = left % size(r);
+      return full % w ? (full / w + 1) * size(r) : full / w * size(r) + part;
     };
-    uint64_t r = std::max<uint64_t>(1, room / w), best = end(1);
-    for (uint64_t k = 2; k <= r; ++k) best = std::min(best, end(k));
-    while (end(r) * 8 > best * 9) --r;
+    uint64_t r = all + 1, best = end(r);
+    for (uint64_t k = 1; k <= all; ++k) best = std::min(best, end(k));
+    while (end(r) * 16 > best * 17) --r;
     I.tail_size = size(r);
     I.rows64 = (int32_t)(used + (left + I.tail_size - 1) / I.tail_size);
     I.rows32 = 0;

@@ -369,7 +369,7 @@ __device__ __forceinline__ void simulate_fd(const PathLaunch& L, const uint4* ta
 // PPT paths per thread, simulated step by step in lockstep: independent
 // dependency chains the scheduler can interleave (instruction-level
 // parallelism at the same occupancy).
-template <bool TAB, int NS, int NV, bool DYN, int PPT, bool QEM = false>
+template <bool TAB, int NS, int NV, bool DYN, int PPT, bool QEM = false, bool ROLL = false>
 __device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint4* tab, const uint64_t (&path)[PPT],
                                              float (&v)[PPT][NS], float (&x)[PPT][NS], float (&c)[PPT][NS]) {
 #pragma unroll
@@ -384,6 +384,28 @@ __device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint4* t
   PhiloxLane pl[PPT];
 #pragma unroll
   for (int j = 0; j < PPT; ++j) pl[j] = philox_lane(path[j], L.rk);
+  if constexpr (ROLL) {  // one step per iteration (path_roll)
+    uint4 w[PPT];
+    uint32_t n = 0;
+    if (NS > 1 && L.first_split) {
+      philox_draws<TAB, PPT>(tab, 0u, L.option_index, L.rk, pl, w);
+#pragma unroll
+      for (int j = 0; j < PPT; ++j) step0_all<NS, DYN, QEM>(L, w[j].x, w[j].y, v[j], x[j], c[j]);
+      n = 1;
+    }
+#pragma unroll 1
+    for (; n < L.steps; ++n) {
+      if (!(n & 1u)) philox_draws<TAB, PPT>(tab, n >> 1, L.option_index, L.rk, pl, w);
+      uint32_t wv[PPT], wx[PPT];
+#pragma unroll
+      for (int j = 0; j < PPT; ++j) {
+        wv[j] = n & 1u ? w[j].z : w[j].x;
+        wx[j] = n & 1u ? w[j].w : w[j].y;
+      }
+      step_paths<NS, NV, DYN, PPT, QEM>(L, wv, wx, v, x, c);
+    }
+    return;
+  }
   const uint32_t pairs = L.steps >> 1;
   uint32_t i0 = 0;
   if (NS > 1 && L.first_split) {
@@ -466,6 +488,17 @@ constexpr bool path_table() {
   return NS == 1 || (NS <= 5 && !QEM);
 }
 
+// Whether simulate_ppt takes one step per iteration: with strike tiles, where the step's
+// code beside the tile's sums overflowed the instruction cache in a long run (four copies of
+// it 208 KB a kernel, one 140 KB: 11 scenarios x 32 strikes, 30 steps x 2.5 M paths 3.2 ->
+// 2.35 ms, 250 steps x 1.05 M paths 4.82 -> 4.30; 7 scenarios the same and 3.50 -> 3.38), and
+// with 11 QE-M scenarios (one strike 5% faster).  One strike under QE keeps two steps, 4%
+// faster at 200 steps with 7 and 11 scenarios, as does the terminal kernel (14%).
+template <int NS, int TILE, bool QEM>
+constexpr bool path_roll() {
+  return TILE > 1 || (QEM && NS >= 11);
+}
+
 // Fused price / Greeks kernel.  TILE = 1 (single strike) or 32 (strike tiles).
 // One block per SM; its warps take the block's batches item by item (ItemPlan).
 // Dynamic shared memory: the strike constants [nk_pad] (StrikeConst), a flag word
@@ -481,7 +514,7 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
   int* s_flag = reinterpret_cast<int*>(ks + L.nk_pad);
   unsigned* s_next = reinterpret_cast<unsigned*>(s_flag + 1);
   uint4* tab = L.pair_table ? reinterpret_cast<uint4*>(s_flag + 4) : nullptr;
-  const ItemRows rows(s_flag + 4 + 4 * L.pair_table, I, L.n_acc * L.nk_pad);
+  const ItemRows rows{smem_raw, (unsigned)(L.nk_pad * sizeof(StrikeConst) + 16 + L.pair_table * sizeof(uint4)), L.n_acc * L.nk_pad};
 
   if (threadIdx.x == 0) *s_next = 0u;
   for (int p = threadIdx.x; p < L.pair_table; p += blockDim.x)
@@ -499,7 +532,7 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
   }
   __syncthreads();
 
-  constexpr bool USE_TAB = path_table<NS, QEM>();
+  constexpr bool USE_TAB = path_table<NS, QEM>(), ROLL = path_roll<NS, TILE, QEM>();
   const uint64_t per_batch = (uint64_t)kWarp * PPT;
   const uint64_t block0 = I.batches / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, I.batches % gridDim.x);
   const uint64_t nb = I.batches / gridDim.x + (blockIdx.x < I.batches % gridDim.x ? 1 : 0);
@@ -510,12 +543,13 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
     uint64_t b0, b1;
     if (!item_range(I, it, nb, b0, b1)) break;
     ItemRow my = rows.at(I, it);
-    for (uint64_t b = b0; b < b1; ++b) {
+    const uint64_t end = (block0 + b1) * per_batch;
+    for (uint64_t first = (block0 + b0) * per_batch; first < end; first += per_batch) {
       uint64_t pth[PPT];
       bool act[PPT];
 #pragma unroll
       for (int j = 0; j < PPT; ++j) {
-        const uint64_t local = (block0 + b) * per_batch + (uint64_t)j * kWarp + lane;
+        const uint64_t local = first + (uint64_t)j * kWarp + lane;
         act[j] = local < L.path_count;
         pth[j] = L.path_begin + local;
       }
@@ -538,9 +572,9 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
         else
           simulate_fd<false, NS, NV>(L, nullptr, pth[0], v[0], x[0], c[0]);
       } else if (USE_TAB && tab) {
-        simulate_ppt<USE_TAB, NS, NV, DYN, PPT, QEM>(L, tab, pth, v, x, c);
+        simulate_ppt<USE_TAB, NS, NV, DYN, PPT, QEM, ROLL>(L, tab, pth, v, x, c);
       } else {
-        simulate_ppt<false, NS, NV, DYN, PPT, QEM>(L, nullptr, pth, v, x, c);
+        simulate_ppt<false, NS, NV, DYN, PPT, QEM, ROLL>(L, nullptr, pth, v, x, c);
       }
       float S[PPT][NS];
 #pragma unroll
@@ -562,7 +596,7 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
             t += act[j] ? tj : 0.0f;
           }
           t = warp_sum(t);
-          if (lane == 0) my.add(a, t);
+          if (lane == 0) my.add<true>(smem_raw, a, t);
         } else {
           for (int t0 = 0; t0 < L.nk_pad; t0 += 32) {
             float vals[32];
@@ -578,22 +612,22 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
               vals[jj] = t;
             }
             butterfly32(vals, lane);
-            my.add(a * L.nk_pad + t0 + lane, vals[0]);
+            my.add<true>(smem_raw, a * L.nk_pad + t0 + lane, vals[0]);
           }
         }
         if (resim) ++r;
         ++a;
       }
-      my.first = false;
+      my.next_batch();
     }
   }
   __syncthreads();
   sum_item_rows(rows, I, nb);
   __syncthreads();
-  if (!sum_block_rows(rows.acc, rows.row, partials, ticket, s_flag)) return;
+  if (!sum_block_rows(rows.acc(I), rows.row, partials, ticket, s_flag)) return;
   for (int k = threadIdx.x; k < L.n_strikes; k += blockDim.x) {
     const double K = strikes[k];
-    write_results(L, k, rows.acc + k, L.nk_pad, out, !(K > 0.0) || !isfinite(K));
+    write_results(L, k, rows.acc(I) + k, L.nk_pad, out, !(K > 0.0) || !isfinite(K));
   }
 }
 
@@ -626,7 +660,13 @@ cudaError_t launch_t(const PathLaunch& L0, const double* strikes, const PathOutp
   const size_t head = L.nk_pad * sizeof(StrikeConst) + 16 + L.pair_table * sizeof(uint4);
   const uint64_t batches = (L.path_count + (uint64_t)kWarp * PPT - 1) / ((uint64_t)kWarp * PPT);
   const uint64_t grid = std::min<uint64_t>(num_sms, batches);  // one block per SM
-  const ItemPlan I = make_item_plan(batches, grid, path_warps<NS, QEM>(), row, kItemBytes - head);
+  ItemPlan I = make_item_plan(batches, grid, path_warps<NS, QEM>(), row, kItemBytes - head);
+  // rows so long that each warp has one fixed share: pricing, whose long strike loop is
+  // issue-bound, with as many warps on every SM sub-partition (50 steps x 2^20 x 768 strikes
+  // 747 -> 688 us at 12 warps for 15, QE-M 803 -> 736; 2^22 x 1,024 strikes 3.75 -> 3.57 ms at
+  // 8 for 10; the bumps and the adjoint lose 3-10% with fewer)
+  if (NS == 1 && I.levels == 0 && I.tail_size > 1 && I.warps > 8 && I.warps % 4)
+    I = make_item_plan(batches, grid, I.warps & ~3, row, kItemBytes - head);
   const int tpb = kWarp * I.warps;
   const size_t smem = head + item_rows_bytes(I, row);
   auto kern = heston_paths_kernel<NS, NV, TILE, DYN, PPT, QEM>;

@@ -34,39 +34,54 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // An item's row: the sums of its batches, added in FP64 in batch order -- or, for
-// an item of one batch, that batch's FP32 sums as they are.
+// an item of one batch, that batch's FP32 sums as they are.  (An offset and a word,
+// not pointers: they live through the whole path loop.)
 struct ItemRow {
-  double* wide;   // null for an FP32 row
-  float* narrow;
-  bool first;     // the item's first batch sets the row
-  __device__ __forceinline__ void add(int i, float t) const {
-    if (!wide)
-      narrow[i] = t;
-    else
-      wide[i] = first ? (double)t : wide[i] + (double)t;
+  unsigned at;  // byte offset of the row in dynamic shared memory
+  int kind;     // 0: FP32; 1: FP64, the item's first batch, which sets the row; 2: FP64
+  // ONE_COPY: the kind hidden from the compiler, which else makes a copy of the loops
+  // over the sums for each kind.  In a long run the warps drift out of step, and with two
+  // copies the path kernels of strike tiles (5 scenarios: 210 KB of code, 172 with one) then
+  // missed the instruction cache: 30 steps x 2.5 M paths x 32 strikes, 5 scenarios 1.60 ->
+  // 1.26 ms; pricing at 8 steps x 8.4 M paths x 64 strikes 0.60 -> 0.55.
+  template <bool ONE_COPY>
+  __device__ __forceinline__ void add(unsigned char* smem, int i, float t) const {
+    int k = kind;
+    if (ONE_COPY) asm volatile("" : "+r"(k));
+    if (k == 0) {
+      reinterpret_cast<float*>(smem + at)[i] = t;
+    } else {
+      double* p = reinterpret_cast<double*>(smem + at) + i;
+      *p = k == 1 ? (double)t : *p + (double)t;
+    }
+  }
+  __device__ __forceinline__ void next_batch() {
+    if (kind == 1) kind = 2;
   }
 };
 
-// The shared memory of a block's items: FP64 rows [rows64][row], the block's
-// totals, FP32 rows [rows32][row].
+// The shared memory of a block's items, from byte offset `base`: FP64 rows
+// [rows64][row], the block's totals, FP32 rows [rows32][row].
 struct ItemRows {
-  double* wide;
-  double* acc;
-  float* narrow;
+  unsigned char* smem;
+  unsigned base;
   int row;
-  __device__ __forceinline__ ItemRows(void* smem, const ItemPlan& I, int row_) : row(row_) {
-    wide = reinterpret_cast<double*>(smem);
-    acc = wide + (size_t)I.rows64 * row;
-    narrow = reinterpret_cast<float*>(acc + max(row, (int)blockDim.x));
+  __device__ __forceinline__ unsigned acc_at(const ItemPlan& I) const { return base + (unsigned)(I.rows64 * row) * 8u; }
+  __device__ __forceinline__ unsigned narrow_at(const ItemPlan& I) const {
+    return acc_at(I) + (unsigned)max(row, (int)blockDim.x) * 8u;
   }
+  __device__ __forceinline__ const double* wide() const { return reinterpret_cast<const double*>(smem + base); }
+  __device__ __forceinline__ const float* narrow(const ItemPlan& I) const {
+    return reinterpret_cast<const float*>(smem + narrow_at(I));
+  }
+  __device__ __forceinline__ double* acc(const ItemPlan& I) const { return reinterpret_cast<double*>(smem + acc_at(I)); }
   __device__ __forceinline__ ItemRow at(const ItemPlan& I, uint32_t it) const {
     const uint32_t n64 = I.tail_size == 1 ? (uint32_t)(I.levels * I.warps) : 0xffffffffu;
-    return it < n64 ? ItemRow{wide + (size_t)it * row, nullptr, true}
-                    : ItemRow{nullptr, narrow + (size_t)(it - n64) * row, true};
+    return it < n64 ? ItemRow{base + it * row * 8u, 1} : ItemRow{narrow_at(I) + (it - n64) * row * 4u, 0};
   }
 };
 
-// The rows of a block that owns nb batches, summed into R.acc in item order: with
+// The rows of a block that owns nb batches, summed into R.acc(I) in item order: with
 // fewer columns than threads, groups of threads sum runs of rows side by side
 // first.  All threads; rows complete on entry (after a barrier).
 __device__ __forceinline__ void sum_item_rows(const ItemRows& R, const ItemPlan& I, uint64_t nb) {
@@ -75,21 +90,24 @@ __device__ __forceinline__ void sum_item_rows(const ItemRows& R, const ItemPlan&
   const int n64 = I.tail_size == 1 ? level_items : n;
   const int groups = max(1, min((int)blockDim.x / row, n));
   const int per = (n + groups - 1) / groups;
+  const double* wide = R.wide();
+  const float* narrow = R.narrow(I);
+  double* acc = R.acc(I);
   for (int i = threadIdx.x; i < row * groups; i += blockDim.x) {
     const int g = i / row, col = i - g * row;
     const int r1 = min((g + 1) * per, n);
     double s = 0.0;
     int r = g * per;
-    for (; r < min(r1, n64); ++r) s += R.wide[(size_t)r * row + col];
-    for (; r < r1; ++r) s += (double)R.narrow[(size_t)(r - n64) * row + col];
-    R.acc[i] = s;
+    for (; r < min(r1, n64); ++r) s += wide[(size_t)r * row + col];
+    for (; r < r1; ++r) s += (double)narrow[(size_t)(r - n64) * row + col];
+    acc[i] = s;
   }
   if (groups == 1) return;
   __syncthreads();
   for (int i = threadIdx.x; i < row; i += blockDim.x) {
-    double s = R.acc[i];
-    for (int g = 1; g < groups; ++g) s += R.acc[g * row + i];
-    R.acc[i] = s;
+    double s = acc[i];
+    for (int g = 1; g < groups; ++g) s += acc[g * row + i];
+    acc[i] = s;
   }
 }
 
