@@ -17,6 +17,7 @@
 
 #include "simr.h"
 #include "simr_internal.h"
+#include "simr_ticket.h"
 
 using namespace simr;
 
@@ -26,9 +27,7 @@ struct simr_ctx {
   // path-kernel scratch: partial rows + ticket
   double* partials = nullptr;
   size_t partial_doubles = 0;
-  // 256-byte block: ticket word at 0, status word at 64, batch queue counter at
-  // 128, Longstaff-Schwartz ticket at 192, its sweep barrier counter at 208
-  unsigned int* ticket = nullptr;
+  unsigned int* ticket = nullptr;  // the counters and the status word (simr_ticket.h)
   int scheme = SIMR_SCHEME_QE;  // log-spot scheme of the path simulations (simr_set_scheme)
   float* ckpt = nullptr;  // adjoint checkpoints, [slot][resident thread]
   size_t ckpt_floats = 0;
@@ -863,9 +862,9 @@ int simr_create(simr_ctx** out, int device) {
   std::snprintf(c->gpu_name, sizeof(c->gpu_name), "%s", prop.name);
   for (char* q = c->gpu_name; *q; ++q)
     if (*q == '"' || *q == '\\') *q = '_';  // kept out of the cache file's strings
-  e = cudaMalloc((void**)&c->ticket, 256);
-  if (e == cudaSuccess) e = cudaMemset(c->ticket, 0, 256);
-  c->status = reinterpret_cast<int*>(reinterpret_cast<char*>(c->ticket) + 64);
+  e = cudaMalloc((void**)&c->ticket, kTicketBytes);
+  if (e == cudaSuccess) e = cudaMemset(c->ticket, 0, kTicketBytes);
+  c->status = reinterpret_cast<int*>(c->ticket + kStatusAt / sizeof(unsigned int));
   if (e != cudaSuccess) {
     cudaFree(c->ticket);
     delete c;
@@ -1337,7 +1336,7 @@ int simr_batch_submit(simr_ctx* ctx, const simr_option* opts, int n_opts, uint64
       e = prepare_batch(B);
       if (e == cudaSuccess) e = cudaEventRecord(a, st);
       if (e == cudaSuccess)
-        e = take_fault(SIMR_FAULT_LAUNCH) ? cudaErrorLaunchOutOfResources : launch_batch(B, ctx->b_opts, ctx->b_items, ctx->ticket + 32, ctx->b_partials, out, ctx->num_sms, st);
+        e = take_fault(SIMR_FAULT_LAUNCH) ? cudaErrorLaunchOutOfResources : launch_batch(B, ctx->b_opts, ctx->b_items, ctx->ticket + kQueueAt / sizeof(unsigned int), ctx->b_partials, out, ctx->num_sms, st);
       if (e == cudaSuccess) e = cudaEventRecord(b, st);
       if (e == cudaSuccess) e = cudaEventSynchronize(b);
       if (e == cudaSuccess) e = cudaEventElapsedTime(ms, a, b);
@@ -1372,7 +1371,7 @@ int simr_batch_submit(simr_ctx* ctx, const simr_option* opts, int n_opts, uint64
   if ((rc = upload_batch(ctx, bo, order, chunk, st, &n_items))) return rc;
   B.n_items = n_items;
   if ((rc = ensure(&ctx->b_partials, &ctx->b_partials_cap, (size_t)n_items * nacc, "batch partial rows"))) return rc;
-  unsigned int* counter = ctx->ticket + 32;  // word at byte 128 of the ticket block
+  unsigned int* counter = ctx->ticket + kQueueAt / sizeof(unsigned int);
   if (flags & SIMR_BATCH_GRAPH) {
     // one captured graph per (book, seed, flags, outputs): repeated submissions replay it.
     // Captured and launched on the context's own stream, ordered after `st` by events
@@ -1714,7 +1713,7 @@ int simr_lsm_price(simr_ctx* ctx, const simr_heston* model, double K, int is_put
                ctx->lsm_xform,
                ctx->lsm_dpow,
                ctx->partials,
-               ctx->ticket + 48,
+               ctx->ticket + kLsmTicketAt / sizeof(unsigned int),
                ctx->status,
                o.dev[0],
                o.dev[1]};

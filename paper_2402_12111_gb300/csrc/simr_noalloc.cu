@@ -16,12 +16,13 @@
 
 #include "simr.h"
 #include "simr_internal.h"
+#include "simr_ticket.h"
 
 namespace {
 
 constexpr int kNoAllocMaxStrikes = 32;
 constexpr int kNoAllocMaxBlocks = 2048;  // blocks of the persistent grid, any SM count up to 256
-constexpr size_t kHeaderBytes = 256;      // ticket word at 0, status word at 64
+constexpr size_t kHeaderBytes = simr::kTicketBytes;
 constexpr size_t kPartialDoubles = (size_t)kNoAllocMaxBlocks * 2 * kNoAllocMaxStrikes;
 constexpr int kMaxDevices = 64;
 
@@ -97,14 +98,14 @@ extern "C" SIMR_API int simr_price_noalloc(const simr_heston* model, const doubl
   if ((rc = simr::internal_build_price_launch(model, n_strikes, is_put, steps, paths, seed, option_index, &L)))
     return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  unsigned int* ticket = reinterpret_cast<unsigned int*>(slot->base);
+  unsigned int* ticket = reinterpret_cast<unsigned int*>(slot->base + simr::kTicketsAt);
   // the ticket and status words must start at zero; the array keeps the last call's contents
   e = cudaMemsetAsync(slot->base, 0, kHeaderBytes, st);
   if (e != cudaSuccess) return simr::internal_cuda_fail(e, "clearing the static scratch header");
   simr::PathOutputs out{};
   out.price = price;
   out.stderr_ = stderr_out;
-  out.status = reinterpret_cast<int*>(slot->base + 64);
+  out.status = reinterpret_cast<int*>(slot->base + simr::kStatusAt);
   simr::Scratch s{reinterpret_cast<double*>(slot->base + kHeaderBytes), ticket, kPartialDoubles};
   int grid = 0;
   e = simr::take_fault(SIMR_FAULT_LAUNCH) ? cudaErrorLaunchOutOfResources
