@@ -115,9 +115,12 @@ __device__ __forceinline__ void write_adjoint(const PathLaunch& L, const AdjCons
   }
 }
 
-// Minimum resident blocks per SM asked of the register allocator: 4, which is what
-// the segment buffers (12 k bytes per thread) leave room for from k = 16 on (11%
-// faster at k = 32 and 1% at k = 16 than with 5).
+// Minimum resident blocks per SM asked of the register allocator: 4 for strike tiles,
+// whose segments (12 k bytes per thread) and rows leave room for no more from k = 16
+// on (11% faster at k = 32 and 1% at k = 16 than with 5); one strike takes 5 where its
+// segments leave room for them, k <= 28 (one_strike_blocks; 96 registers instead of 108:
+// QE-M 9 steps x 2^22 paths 825 -> 748 us, 96 steps at k = 16 5.12 -> 4.82 ms), else 4
+// (1% faster at k = 32 and 64).
 #ifndef SIMR_ADJ_MINB_SMEM
 #define SIMR_ADJ_MINB_SMEM 4
 #endif
@@ -125,8 +128,8 @@ __device__ __forceinline__ void write_adjoint(const PathLaunch& L, const AdjCons
 // Segments in shared memory (an explicit checkpoint interval).
 // QEM: the QE-M log-spot step (the launch's scheme 1), differentiated one step
 // at a time.
-template <int TILE, int PPT, bool RACC, bool QEM>
-__global__ void __launch_bounds__(128, SIMR_ADJ_MINB_SMEM) heston_adjoint_kernel(const __grid_constant__ PathLaunch L,
+template <int TILE, int PPT, bool RACC, bool QEM, int MINB = SIMR_ADJ_MINB_SMEM>
+__global__ void __launch_bounds__(128, MINB) heston_adjoint_kernel(const __grid_constant__ PathLaunch L,
                                                              const __grid_constant__ AdjConst A,
                                                              const double* __restrict__ strikes, AdjOutputs out,
                                                              double* __restrict__ partials,
@@ -337,14 +340,20 @@ __global__ void __launch_bounds__(128) heston_paths_adjoint_kernel(const __grid_
   for (int j = 0; j < 5; ++j) grad[i * 5 + j] = g[0][j];
 }
 
-template <int TILE, bool RACC, bool QEM>
+// Blocks per SM that one strike's segments leave room for, 5 at most and 4 at least
+// (an SM's shared memory less 1 KB per block).
+int one_strike_blocks(const PathLaunch& L, const AdjConst& A) {
+  return 5 * (adjoint_smem_bytes_t(L, A, 128, SIMR_ADJ_PPT, false) + 1024) <= 228 * 1024 ? 5 : 4;
+}
+
+template <int TILE, bool RACC, bool QEM, int MINB = SIMR_ADJ_MINB_SMEM>
 cudaError_t launch_adjoint_t(const PathLaunch& L, const AdjConst& A, const double* strikes, const AdjOutputs& out,
                              const Scratch& s, int num_sms, cudaStream_t stream) {
   constexpr int PPT = SIMR_ADJ_PPT;
   const int tpb = 128, warps = tpb / kWarp;
   const size_t row = (size_t)kAdjAcc * L.nk_pad;
   const size_t smem = adjoint_smem_bytes_t(L, A, tpb, PPT, RACC);
-  auto kern = heston_adjoint_kernel<TILE, PPT, RACC, QEM>;
+  auto kern = heston_adjoint_kernel<TILE, PPT, RACC, QEM, MINB>;
   cudaError_t e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
@@ -412,7 +421,9 @@ cudaError_t launch_adjoint_s(const PathLaunch& L, const AdjConst& A, const doubl
     return L.nk_pad == 1 ? launch_adjoint_seg<1, QEM>(L, A, strikes, out, s, num_sms, stream)
                          : launch_adjoint_seg<32, QEM>(L, A, strikes, out, s, num_sms, stream);
   }
-  if (L.nk_pad == 1) return launch_adjoint_t<1, false, QEM>(L, A, strikes, out, s, num_sms, stream);
+  if (L.nk_pad == 1)
+    return one_strike_blocks(L, A) == 5 ? launch_adjoint_t<1, false, QEM, 5>(L, A, strikes, out, s, num_sms, stream)
+                                        : launch_adjoint_t<1, false, QEM>(L, A, strikes, out, s, num_sms, stream);
   if (L.nk_pad == 32) return launch_adjoint_t<32, true, QEM>(L, A, strikes, out, s, num_sms, stream);
   return launch_adjoint_t<32, false, QEM>(L, A, strikes, out, s, num_sms, stream);
 }
