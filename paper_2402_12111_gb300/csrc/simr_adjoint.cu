@@ -38,16 +38,14 @@ namespace {
 #ifndef SIMR_ADJ_PPT
 #define SIMR_ADJ_PPT 1  // paths per thread of the per-strike adjoint kernel (2 measured slower)
 #endif
-// Dynamic shared memory of the per-strike kernel: strike constants, the
-// last-block flag, then the segment buffers (none when they are in global
-// memory, GSEG); the per-warp FP64 accumulator rows come first when they live in
-// shared memory throughout (RACC false), or reuse the segment buffers' space
-// once the path loop has ended (RACC true: lane l accumulates strike l of the
-// one 32-strike tile in registers).
-inline size_t adjoint_smem_bytes_t(const PathLaunch& L, const AdjConst& A, int tpb, int ppt, bool racc,
-                                   bool gseg = false) {
+// Dynamic shared memory of the per-strike kernel with segments in shared memory: strike
+// constants, the last-block flag, then the segment buffers; the per-warp FP64 accumulator
+// rows come first when they live in shared memory throughout (RACC false), or reuse the
+// segment buffers' space once the path loop has ended (RACC true: lane l accumulates strike
+// l of the one 32-strike tile in registers).
+inline size_t adjoint_smem_bytes_t(const PathLaunch& L, const AdjConst& A, int tpb, int ppt, bool racc) {
   const size_t acc_bytes = (size_t)(tpb / kWarp) * kAdjAcc * L.nk_pad * sizeof(double);
-  const size_t buf_bytes = gseg ? 0 : adjoint_seg_floats(A, ppt) * tpb * sizeof(float);
+  const size_t buf_bytes = adjoint_seg_floats(A, ppt) * tpb * sizeof(float);
   const size_t head = L.nk_pad * sizeof(StrikeConst) + 16;
   return racc ? head + (buf_bytes > acc_bytes ? buf_bytes : acc_bytes) : acc_bytes + head + buf_bytes;
 }
@@ -465,10 +463,6 @@ cudaError_t adjoint_max_ckpt_every(const PathLaunch& L, int steps_cap, int* k_ma
   }
   *k_max = 2 * lo;
   return cudaSuccess;
-}
-
-size_t adjoint_smem_bytes(const PathLaunch& L, const AdjConst& A) {
-  return adjoint_smem_bytes_t(L, A, 128, SIMR_ADJ_PPT, L.nk_pad == 32, adjoint_gseg(L, A));
 }
 
 cudaError_t adjoint_gseg_floats(const PathLaunch& L, const AdjConst& A, int num_sms, size_t* floats) {

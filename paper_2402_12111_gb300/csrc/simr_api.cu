@@ -1048,9 +1048,8 @@ int simr_greeks_adjoint(simr_ctx* ctx, const simr_heston* model, const double* s
   AdjConst A;
   if ((rc = build_adjoint(*model, steps, k, &A))) return rc;
   adjoint_scheme(ctx, *model, steps, &L, &A);
-  if (adjoint_smem_bytes(L, A) > kAdjMaxSmem)
-    return fail(SIMR_EUNSUPPORTED, "ckpt_every %d with %u steps needs more shared memory than a block has",
-                A.ckpt_every, steps);
+  // (shared memory needs no check: segments past kAdjMaxSmem go to global memory, and the
+  // item plan keeps that kernel's rows within kItemBytes)
   if (adjoint_ckpt_scratch_floats(A, ctx->num_sms) > (1ull << 30))
     return fail(SIMR_EUNSUPPORTED, "ckpt_every %d with %u steps gives more than 2^30 checkpoint floats",
                 A.ckpt_every, steps);

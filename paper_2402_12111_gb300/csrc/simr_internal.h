@@ -185,7 +185,6 @@ cudaError_t launch_finalize(const PathLaunch& L, const double* sums, const PathO
 cudaError_t launch_adjoint(const PathLaunch& L, const AdjConst& A, const double* strikes, const AdjOutputs& out,
                            const Scratch& s, int num_sms, cudaStream_t stream);
 size_t adjoint_scratch_doubles(const PathLaunch& L, int num_sms);
-size_t adjoint_smem_bytes(const PathLaunch& L, const AdjConst& A);
 // Dynamic shared memory one block of an adjoint kernel may ask for.
 constexpr size_t kAdjMaxSmem = 200 * 1024;
 // Largest global segment buffer of the per-strike adjoint (8 GB), and the
