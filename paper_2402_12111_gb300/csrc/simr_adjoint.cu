@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kWarp * (QEM ? SIMR_ADJ_QEM_WARPS : SIMR_ADJ_W
     it = __shfl_sync(kFull, it, 0);
     uint64_t b0, b1;
     if (!item_range(I, it, nb, b0, b1)) break;
-    ItemRow my = rows.at(I, it);
+    ItemRow<false> my = rows.at(I, it);
     for (uint64_t b = b0; b < b1; ++b) {
       const uint64_t local = (block0 + b) * kWarp + lane;
       const bool act[1] = {local < L.path_count};

@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kWarp * basket_warps<NA>(), 1)
     it = __shfl_sync(kFull, it, 0);
     uint64_t b0, b1;
     if (!item_range(I, it, nb, b0, b1)) break;
-    ItemRow my = rows.at(I, it);
+    ItemRow<false> my = rows.at(I, it);
     for (uint64_t b = b0; b < b1; ++b) {
       const uint64_t path = (block0 + b) * kWarp + lane;
       const bool active = path < L.paths;

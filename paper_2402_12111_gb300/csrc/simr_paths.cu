@@ -499,6 +499,15 @@ constexpr bool path_roll() {
   return TILE > 1 || (QEM && NS >= 11);
 }
 
+// The form of an item's row (ItemRow): pointers for QE pricing (252 steps x 2^20 paths x 32
+// strikes 741 us, 748 with an offset) and 11 scenarios (365 x 250,001 x 21 1,619 / 1,667 us);
+// an offset for 5 scenarios (252 x 2^20 x 32 2,160 us with pointers, 2,132 with it), 3 (64 x
+// 65,536 88.9 / 86.6) and QE-M (pricing 1% slower with pointers).
+template <int NS, bool QEM>
+constexpr bool path_row_pointers() {
+  return !QEM && (NS == 1 || NS == 11);
+}
+
 // Fused price / Greeks kernel.  TILE = 1 (single strike) or 32 (strike tiles).
 // One block per SM; its warps take the block's batches item by item (ItemPlan).
 // Dynamic shared memory: the strike constants [nk_pad] (StrikeConst), a flag word
@@ -542,7 +551,7 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
     it = __shfl_sync(kFull, it, 0);
     uint64_t b0, b1;
     if (!item_range(I, it, nb, b0, b1)) break;
-    ItemRow my = rows.at(I, it);
+    auto my = rows.template at<path_row_pointers<NS, QEM>()>(I, it);
     const uint64_t end = (block0 + b1) * per_batch;
     for (uint64_t first = (block0 + b0) * per_batch; first < end; first += per_batch) {
       uint64_t pth[PPT];

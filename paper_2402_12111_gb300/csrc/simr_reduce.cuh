@@ -34,16 +34,18 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // An item's row: the sums of its batches, added in FP64 in batch order -- or, for
-// an item of one batch, that batch's FP32 sums as they are.  (An offset and a word,
-// not pointers: they live through the whole path loop.)
+// an item of one batch, that batch's FP32 sums as they are.  It lives through the whole
+// path loop, as an offset and a word or as pointers and a flag: which of the two leaves a
+// kernel the better schedule is measured (path_row_pointers).
+// ONE_COPY: the row's kind hidden from the compiler, which else makes a copy of the loops
+// over the sums for each kind.  In a long run the warps drift out of step, and with two
+// copies the path kernels of strike tiles (5 scenarios: 210 KB of code, 172 with one) then
+// missed the instruction cache: 30 steps x 2.5 M paths x 32 strikes, 5 scenarios 1.60 ->
+// 1.26 ms; pricing at 8 steps x 8.4 M paths x 64 strikes 0.60 -> 0.55.
+template <bool POINTERS>
 struct ItemRow {
   unsigned at;  // byte offset of the row in dynamic shared memory
   int kind;     // 0: FP32; 1: FP64, the item's first batch, which sets the row; 2: FP64
-  // ONE_COPY: the kind hidden from the compiler, which else makes a copy of the loops
-  // over the sums for each kind.  In a long run the warps drift out of step, and with two
-  // copies the path kernels of strike tiles (5 scenarios: 210 KB of code, 172 with one) then
-  // missed the instruction cache: 30 steps x 2.5 M paths x 32 strikes, 5 scenarios 1.60 ->
-  // 1.26 ms; pricing at 8 steps x 8.4 M paths x 64 strikes 0.60 -> 0.55.
   template <bool ONE_COPY>
   __device__ __forceinline__ void add(unsigned char* smem, int i, float t) const {
     int k = kind;
@@ -58,6 +60,22 @@ struct ItemRow {
   __device__ __forceinline__ void next_batch() {
     if (kind == 1) kind = 2;
   }
+};
+template <>
+struct ItemRow<true> {
+  double* wide;   // null for an FP32 row
+  float* narrow;
+  bool first;     // the item's first batch sets the row
+  template <bool ONE_COPY>
+  __device__ __forceinline__ void add(unsigned char*, int i, float t) const {
+    int w = wide != nullptr;
+    if (ONE_COPY) asm volatile("" : "+r"(w));
+    if (!w)
+      narrow[i] = t;
+    else
+      wide[i] = first ? (double)t : wide[i] + (double)t;
+  }
+  __device__ __forceinline__ void next_batch() { first = false; }
 };
 
 // The shared memory of a block's items, from byte offset `base`: FP64 rows
@@ -75,9 +93,14 @@ struct ItemRows {
     return reinterpret_cast<const float*>(smem + narrow_at(I));
   }
   __device__ __forceinline__ double* acc(const ItemPlan& I) const { return reinterpret_cast<double*>(smem + acc_at(I)); }
-  __device__ __forceinline__ ItemRow at(const ItemPlan& I, uint32_t it) const {
+  template <bool POINTERS = false>
+  __device__ __forceinline__ ItemRow<POINTERS> at(const ItemPlan& I, uint32_t it) const {
     const uint32_t n64 = I.tail_size == 1 ? (uint32_t)(I.levels * I.warps) : 0xffffffffu;
-    return it < n64 ? ItemRow{base + it * row * 8u, 1} : ItemRow{narrow_at(I) + (it - n64) * row * 4u, 0};
+    if constexpr (POINTERS)
+      return it < n64 ? ItemRow<true>{reinterpret_cast<double*>(smem + base) + (size_t)it * row, nullptr, true}
+                      : ItemRow<true>{nullptr, reinterpret_cast<float*>(smem + narrow_at(I)) + (size_t)(it - n64) * row, true};
+    else
+      return it < n64 ? ItemRow<false>{base + it * row * 8u, 1} : ItemRow<false>{narrow_at(I) + (it - n64) * row * 4u, 0};
   }
 };
 
