@@ -6,7 +6,7 @@
 // reverse sweep over the segments, last to first: each segment's states are
 // recomputed from its checkpoint (the draws are counter-based, so the
 // segment's draws are regenerated) and kept with the step's branch draw and Z_X
-// -- in shared memory, or in a global [3 k][resident thread] buffer when the
+// -- in shared memory, or in a slab per warp in global memory (SegWarp) when the
 // segment is longer than shared memory holds -- and the steps are
 // differentiated backwards (LogPricePathQE's increments summed on the way),
 // with the branch taken in the forward pass held fixed (pathwise derivative).
@@ -233,10 +233,10 @@ __global__ void __launch_bounds__(128, MINB) heston_adjoint_kernel(const __grid_
 #define SIMR_ADJ_QEM_WARPS 28
 #endif
 
-// Segments in global memory, [3 k][grid threads] (a segment too long for shared
+// Segments in global memory, a slab per warp of 3 k floats a lane (a segment too long for shared
 // memory, in particular one segment of the whole path: no forward pass).  One block
 // per SM, its warps taking 32-path batches item by item (ItemPlan), each item's nine
-// sums per strike in the item's own row.  Issue-bound (187 warp instructions per
+// sums per strike in the item's own row.  Issue-bound (152 warp instructions per
 // path-step, 33 of them packed).  252 steps x 2^20 paths x 32 strikes: 2,072 us with
 // five blocks of 128 that strode over the batches (and one thread per sum over 760
 // block rows at the end), 1,740 with items at 20 warps, 1,598 at 24 (80 registers;

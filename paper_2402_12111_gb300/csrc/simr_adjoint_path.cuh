@@ -524,8 +524,8 @@ __device__ __forceinline__ void keep_step(const ScenConst& c, float xv, float zv
 }
 
 // A segment's stored steps, in pairs (2p, 2p + 1): each step's (state, branch draw)
-// as one float2 and the pair's two Z_X as another, three float2 rows kRow apart per
-// pair and pairs kPair rows apart.  SegShared: the block's buffer in shared memory,
+// as one float2 and the pair's two Z_X as another, three rows of float2 per
+// pair, row() apart, and the pairs three rows apart.  SegShared: the block's buffer in shared memory,
 // one column per thread.  SegWarp: the warp's own slab in global memory, [pair][3][32
 // lanes] -- a warp's accesses are contiguous and every offset is a constant, where a
 // grid-wide [step][thread] array cost eight 64-bit address sums per step.

@@ -31,7 +31,7 @@ struct simr_ctx {
   int scheme = SIMR_SCHEME_QE;  // log-spot scheme of the path simulations (simr_set_scheme)
   float* ckpt = nullptr;  // adjoint checkpoints, [slot][resident thread]
   size_t ckpt_floats = 0;
-  float* gseg = nullptr;  // adjoint segment buffers too long for shared memory, [3 k][resident thread]
+  float* gseg = nullptr;  // adjoint segment buffers too long for shared memory, a slab per resident warp
   size_t gseg_floats = 0;
   // Longstaff-Schwartz: states at the exercise dates, per-path cash flows,
   // coefficients, discount table

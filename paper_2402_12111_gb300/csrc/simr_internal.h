@@ -127,7 +127,7 @@ struct BatchLaunch {
   int32_t adjoint;
   int32_t ckpt_rows;  // adjoint: checkpoint rows per thread column (max over options of n_seg - 1), even
   int32_t seg_rows;   // adjoint: rows of each segment array (max over options of ckpt_every)
-  float* gseg;        // adjoint with one segment per path: [3 seg_rows][grid threads] in global memory, else null
+  float* gseg;        // adjoint with one segment per path: a slab per warp in global memory (SegWarp), else null
   size_t gseg_floats;  // its capacity
   int32_t tab_rows;    // entries of each warp's step-pair counter table, 0: none (shared segments have none)
   int32_t tpb, ppt, unroll;  // the kernel's shape (batch_variant)

@@ -23,7 +23,9 @@
 // average, and one thread per sum then added 608 rows.  Items taken from a
 // counter and the two-level sums: pricing 252 steps x 2^20 paths x 32 strikes
 // 885 -> 780 us, the 5-scenario Greeks 2,510 -> 2,270 us, one strike's delta,
-// gamma and vega at 64 x 65,536 52.7 -> 43.5 us (warm calls back to back).
+// gamma and vega at 64 x 65,536 52.7 -> 43.5 us (warm calls back to back).  Rows too
+// long for several a warp (from 128 strikes x 7 sums on, and sooner for long runs)
+// leave each warp one or two long items, a fixed share in all but name.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -36,8 +38,10 @@
 // Tuning knobs (compile-time): warps per SM.  Measured at 252 steps x 2^20 paths:
 // pricing 770 / 785 / 786 us at 24 / 28 / 32 warps (pipelined loops); 5 scenarios
 // 2,138 / 2,170 us at 24 / 28; 11 scenarios (365 x 250,001) 1,707 / 1,728 / 1,918 us at
-// 16 / 20 / 24; 3 scenarios (one strike, 64 x 65,536) 39 us at 20 and 24.  QE-M pricing 285 / 289 / 242 us at 24 /
-// 28 / 32 (101 x 300,007 x 40 strikes: 31 batches a block), before the pipelined loop.
+// 16 / 20 / 24; 3 scenarios (one strike, 64 x 65,536) 39 us at 20 and 24.  QE-M pricing x 32
+// strikes at 24 / 28 / 32: 252 x 2^20 940 / 926 / 942 us on the base model and 1,595 / 1,539 /
+// 1,541 at a Feller ratio of 0.04, there 252 x 2^22 5,887 / 5,774 / 5,670 and 101 x 300,007 (31
+// batches a block) 265 / 265 / 233.
 #ifndef SIMR_PRICE_WARPS
 #define SIMR_PRICE_WARPS 24
 #endif
@@ -384,7 +388,7 @@ __device__ __forceinline__ void simulate_ppt(const PathLaunch& L, const uint4* t
   PhiloxLane pl[PPT];
 #pragma unroll
   for (int j = 0; j < PPT; ++j) pl[j] = philox_lane(path[j], L.rk);
-  if constexpr (ROLL) {  // one step per iteration (path_roll)
+  if constexpr (ROLL) {  // one step per iteration (path_roll_steps)
     uint4 w[PPT];
     uint32_t n = 0;
     if (NS > 1 && L.first_split) {
@@ -488,15 +492,17 @@ constexpr bool path_table() {
   return NS == 1 || (NS <= 5 && !QEM);
 }
 
-// Whether simulate_ppt takes one step per iteration: with strike tiles, where the step's
-// code beside the tile's sums overflowed the instruction cache in a long run (four copies of
-// it 208 KB a kernel, one 140 KB: 11 scenarios x 32 strikes, 30 steps x 2.5 M paths 3.2 ->
-// 2.35 ms, 250 steps x 1.05 M paths 4.82 -> 4.30; 7 scenarios the same and 3.50 -> 3.38), and
-// with 11 QE-M scenarios (one strike 5% faster).  One strike under QE keeps two steps, 4%
+// The steps up to which simulate_ppt takes one step per iteration: all with strike tiles,
+// where the step's code beside the tile's sums overflowed the instruction cache in a long run
+// (four copies of it 208 KB a kernel, one 140 KB: 11 scenarios x 32 strikes, 30 steps x 2.5 M
+// paths 3.2 -> 2.35 ms, 250 steps x 2^22 paths 18.8 -> 16.8; 13 scenarios 4% faster at 1,024
+// steps still), but for 11 QE scenarios, where two steps an iteration win once the steps
+// outweigh the sums (1,024 x 2^22 64.05 / 62.05 ms, 500 x 2^20 8.11 / 8.40, even near 760);
+// and with 11 QE-M scenarios (one strike 5% faster).  One strike under QE keeps two steps, 4%
 // faster at 200 steps with 7 and 11 scenarios, as does the terminal kernel (14%).
 template <int NS, int TILE, bool QEM>
-constexpr bool path_roll() {
-  return TILE > 1 || (QEM && NS >= 11);
+constexpr uint32_t path_roll_steps() {
+  return NS == 11 && TILE > 1 && !QEM ? 760u : TILE > 1 || (QEM && NS >= 11) ? 0xffffffffu : 0u;
 }
 
 // The form of an item's row (ItemRow): pointers for QE pricing (252 steps x 2^20 paths x 32
@@ -512,7 +518,7 @@ constexpr bool path_row_pointers() {
 // One block per SM; its warps take the block's batches item by item (ItemPlan).
 // Dynamic shared memory: the strike constants [nk_pad] (StrikeConst), a flag word
 // and the item counter, the step pairs' counter table, then the items' rows of n_acc x nk_pad sums (ItemRows).
-template <int NS, int NV, int TILE, bool DYN, int PPT, bool QEM>
+template <int NS, int NV, int TILE, bool DYN, int PPT, bool QEM, bool ROLL>
 __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
     heston_paths_kernel(const __grid_constant__ PathLaunch L, const __grid_constant__ ItemPlan I,
                         const double* __restrict__ strikes, PathOutputs out, double* __restrict__ partials,
@@ -541,7 +547,7 @@ __global__ void __launch_bounds__(kWarp * path_warps<NS, QEM>(), 1)
   }
   __syncthreads();
 
-  constexpr bool USE_TAB = path_table<NS, QEM>(), ROLL = path_roll<NS, TILE, QEM>();
+  constexpr bool USE_TAB = path_table<NS, QEM>();
   const uint64_t per_batch = (uint64_t)kWarp * PPT;
   const uint64_t block0 = I.batches / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, I.batches % gridDim.x);
   const uint64_t nb = I.batches / gridDim.x + (blockIdx.x < I.batches % gridDim.x ? 1 : 0);
@@ -678,7 +684,10 @@ cudaError_t launch_t(const PathLaunch& L0, const double* strikes, const PathOutp
     I = make_item_plan(batches, grid, I.warps & ~3, row, kItemBytes - head);
   const int tpb = kWarp * I.warps;
   const size_t smem = head + item_rows_bytes(I, row);
-  auto kern = heston_paths_kernel<NS, NV, TILE, DYN, PPT, QEM>;
+  constexpr uint32_t roll = path_roll_steps<NS, TILE, QEM>();
+  auto kern = heston_paths_kernel<NS, NV, TILE, DYN, PPT, QEM, (roll > 0)>;
+  if constexpr (roll > 0 && roll < 0xffffffffu)
+    if (L.steps > roll) kern = heston_paths_kernel<NS, NV, TILE, DYN, PPT, QEM, false>;
   cudaError_t e = cudaSuccess;
   if (smem > 48 * 1024)  // (below, the default suffices)
     e = allow_dynamic_smem(kern);

@@ -80,6 +80,14 @@ def test_a_strike_alone_equals_the_strike_in_a_grid(simr, steps, scen, split, sc
     _same(grid, [torch.cat([a[i] for a in alone]) for i in range(2)])
 
 
+@pytest.mark.parametrize("steps", [760, 761, 762])
+def test_eleven_scenarios_at_the_step_count_that_changes_the_loop(simr, steps):
+    # a tile of strikes under QE: one step an iteration up to 760 steps, two beyond
+    grid = simr.greeks_fd(CFG, _dev(K3), False, steps, 700, 7, greeks=GREEKS[11], rel_bump=1e-2)
+    alone = [simr.greeks_fd(CFG, _dev([k]), False, steps, 700, 7, greeks=GREEKS[11], rel_bump=1e-2) for k in K3]
+    _same(grid, [torch.cat([a[i] for a in alone]) for i in range(2)])
+
+
 @pytest.mark.parametrize("split", [True, False])
 @pytest.mark.parametrize("n_strikes", [1, 3])
 @pytest.mark.parametrize("scen", [3, 5])
