@@ -39,7 +39,8 @@
  *    copies results back and synchronises `stream` before returning.
  *  - The library never frees caller memory.  Its own device scratch belongs to
  *    the context; calls on one context must not run concurrently on different
- *    streams (they share that scratch).
+ *    streams (they share that scratch).  Different contexts, also of one device,
+ *    may be used by different host threads at the same time.
  *  - Model validity: S0, K, T > 0; v0, theta >= 0; kappa > 0; sigma > 0 (the
  *    log-spot coefficients divide by sigma); rho in [-1, 1]; all finite;
  *    steps >= 1; paths >= 1.
